@@ -159,6 +159,16 @@ int spfm_last_zchunk(const spfm_grid *g);
  * rounds.  Host only, no device call.  -1 for an argument below 1. */
 int spfm_debug_pick_zchunk(int tiles, int nz, int per_sm, int sms, int target);
 
+/* Test hook (the paper has no counterpart): the TI potential's sum over the
+ * coupling groups, sum_k 4 c_k A_k / (1 - A_k (1 - 4 q)) at M = 1, C_Gamma = 2/3
+ * and dt = 1, at n values of q = phi (1 - phi), by the FP64 coefficients of the
+ * form that the step kernels take for grids of this storage type, stencil,
+ * coupling direction u and lambda, dx; below its range group by group, as they
+ * do.  Returns the degree of that form (0: group by group for every q), or -1.
+ * *q_lo (may be NULL) receives its lowest q.  Host only, no device call. */
+int spfm_debug_potential(int dtype, int stencil, const double u[3], double lambda, double dx, int n,
+                         const double *q, double *out, double *q_lo);
+
 /* Test hook of the failure reporting (the paper has no counterpart): the next
  * spfm_step launch skips the copy of one plane in its first CTA, whose bounded
  * waits (about 2 s each) then give up; the kernel returns without writing that

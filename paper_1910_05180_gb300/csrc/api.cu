@@ -104,8 +104,34 @@ int build_model(spfm_grid *g, double M, double Gamma, double lambda, double dx, 
         int t = 0;
         for (; t < m.nterms; ++t)
             if (fabs(m.A[t] - A) <= 4e-15 * A) break;
-        if (t == m.nterms) { m.A[t] = A; m.beta[t] = 0.0; ++m.nterms; }
+        if (t == m.nterms) {
+            m.A[t] = A;
+            m.E[t] = 1.0 - A;
+            // near 1 the difference has lost its digits: sech^2 instead
+            if (m.E[t] < 0.01) {
+                const Dir d = grid_dir(k);
+                const double *u = coupling_dir(g);
+                const double ch = cosh(2.0 * dx * (d.x * u[0] + d.y * u[1] + d.z * u[2]) / lambda);
+                m.E[t] = 1.0 / (ch * ch);
+            }
+            m.beta[t] = 0.0;
+            ++m.nterms;
+        }
         m.beta[t] += beta;
+    }
+    m.rat.deg = 0;
+    if (scheme == SPFM_TI_GLOBAL) {
+        // beta scales with D alone, so the grid's form at D = 1 serves every M
+        if (g->rat_lambda != lambda || g->rat_dx != dx || g->rat_stencil != stencil) {
+            double b1[kMaxTerms];
+            for (int t = 0; t < m.nterms; ++t) b1[t] = m.beta[t] / m.D;
+            build_rational(m.A, m.E, b1, m.nterms, g->d.dtype != SPFM_F64, g->rat);
+            g->rat_lambda = lambda;
+            g->rat_dx = dx;
+            g->rat_stencil = stencil;
+        }
+        m.rat = g->rat;
+        for (int i = 0; i < m.rat.deg; ++i) m.rat.num[i] *= m.D;
     }
     m.kmu = 4.0 * M * dF / (lambda * Gamma);
     m.kappa = m.D / (lambda * lambda) * (16.0 / 3.0) * wsum;
@@ -377,6 +403,33 @@ spfm_status spfm_set_zchunk(spfm_grid *g, int zchunk)
 }
 
 int spfm_last_zchunk(const spfm_grid *g) { return g ? g->last_zchunk : -1; }
+
+int spfm_debug_potential(int dtype, int stencil, const double u[3], double lambda, double dx, int n,
+                         const double *q, double *out, double *q_lo)
+{
+    if (!u || !q || !out || n < 0) return -1;
+    spfm_grid g;
+    memset(&g.d, 0, sizeof g.d);
+    g.d.dtype = dtype;
+    for (int i = 0; i < 3; ++i) g.d.n[i] = g.d.u[i] = u[i];
+    Model m;
+    if (build_model(&g, 1.0, 1.0, lambda, dx, 1e-300, 0.0, stencil, SPFM_TI_GLOBAL, m) != SPFM_OK) return -1;
+    for (int i = 0; i < n; ++i) {
+        if (m.rat.deg == 0 || q[i] < m.rat.q_lo) {
+            out[i] = 0.0;
+            for (int t = 0; t < m.nterms; ++t) out[i] += m.beta[t] / (m.E[t] + 4.0 * m.A[t] * q[i]);
+        } else {
+            double num = 0.0, den = 0.0;
+            for (int k = m.rat.deg; k >= 0; --k) {
+                if (k < m.rat.deg) num = num * q[i] + m.rat.num[k];
+                den = den * q[i] + m.rat.den[k];
+            }
+            out[i] = num / den;
+        }
+    }
+    if (q_lo) *q_lo = m.rat.q_lo;
+    return m.rat.deg;
+}
 
 int spfm_current(const spfm_grid *g) { return g ? g->cur : -1; }
 

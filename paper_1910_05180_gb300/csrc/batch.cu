@@ -11,6 +11,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "host_internal.h"
@@ -301,6 +302,7 @@ spfm_status spfm_batch_step(spfm_batch *b, int n_steps, const spfm_step_args *ar
     const size_t rec = grid_record_bytes(b->dtype);
     cudaError_t e = cudaSuccess;
     b->sr = b->grids[0]->rounding == SPFM_ROUND_STOCHASTIC ? 1 : 0;
+    int kind = 0;   // the step kernel's, for the highest degree of the grids' potentials
     for (int i = 0; i < b->n; ++i) {
         spfm_grid *g = b->grids[i];
         const spfm_step_args &a = args[i];
@@ -324,6 +326,7 @@ spfm_status spfm_batch_step(spfm_batch *b, int n_steps, const spfm_step_args *ar
             g->ghost_lambda = a.lambda;
             g->ghost_dx = a.dx;
         }
+        kind = std::max(kind, grid_kind(scheme, m.rat.deg, false));
         void *slot = b->h_grids.data() + rec * i;
         if (b->dtype == SPFM_F64) {
             StepCoef<double> c;
@@ -343,7 +346,6 @@ spfm_status spfm_batch_step(spfm_batch *b, int n_steps, const spfm_step_args *ar
         gj.cur = g->cur;
     }
     if (n_steps == 0) return SPFM_OK;
-    const int kind = is_fd_scheme(scheme) ? 0 : 5;
     e = cudaMemcpyAsync(b->scratch + b->L.grids, b->h_grids.data(), rec * b->n, cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->scratch + b->L.ghosts, b->h_ghosts.data(), sizeof(GhostJob) * b->n,

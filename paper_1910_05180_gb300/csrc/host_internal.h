@@ -7,6 +7,18 @@
 
 #include "spfm_internal.h"
 
+namespace spfm_host {
+
+// sum_k beta_k / (1 - A_k s^2) as N(q) / D(q) of q = phi (1 - phi): coefficients
+// of q^i (deg of them in N, deg + 1 in D, D(0) = 1), the lowest q it covers
+// (-inf: all).  deg 0: no such form within the FP32 range.
+struct Rational {
+    int deg = 0;
+    double num[spfm::kMaxTerms], den[spfm::kMaxTerms + 1], q_lo;
+};
+
+}  // namespace spfm_host
+
 struct spfm_grid {
     spfm_grid_desc d;
     spfm::GridGeom geom;
@@ -26,6 +38,11 @@ struct spfm_grid {
     bool skip_copy = false;   // spfm_debug_skip_copy: the next step launch skips one copy
     int zchunk = 0;           // spfm_set_zchunk: planes per CTA of the step launches (0: chosen per launch)
     int last_zchunk = 0;      // planes per CTA of the last step launch
+    // N / D of the TI potential for these lambda, dx and stencil, at D = 1
+    // (build_model scales it); the groups follow from the descriptor's u, n and gamma
+    spfm_host::Rational rat;
+    double rat_lambda = 0.0, rat_dx = 0.0;
+    int rat_stencil = 0;
     std::string err;
 };
 
@@ -42,11 +59,16 @@ int check_extent(const spfm_grid_desc *d, size_t pitch_x, const char *who);
 
 // Model coefficients in FP64 (a1).  gamma defaults, nu_j = 3/m_j, c_j, A_k
 // grouped by value, stability and phase checks.
+// From K groups with A_k, E_k = 1 - A_k and beta_k (potential.cu).  fewer: as
+// few terms as keep the sum to 2^-30 (FP32 compute); else all K.
+void build_rational(const double *A, const double *E, const double *beta, int K, bool fewer, Rational &r);
+
 struct Model {
     double gamma[3], w[spfm::kMaxTerms], c_shell[3], ck[spfm::kMaxTerms];
     double a[spfm::kMaxTerms];
     int nterms;
-    double beta[spfm::kMaxTerms], A[spfm::kMaxTerms];
+    double beta[spfm::kMaxTerms], A[spfm::kMaxTerms], E[spfm::kMaxTerms];   // E = 1 - A
+    Rational rat;   // of the groups, for the grid's compute type (TI global)
     double kmu, kappa, D, Cg;
     int interp;     // CF driving term: 0 h3, 1 h5, 2 h_Abel
     double aface[6];
@@ -88,6 +110,10 @@ void fill_coef(const spfm_grid *g, const Model &m, double dt, int stencil, spfm:
         c.ck[t] = (T)m.ck[t];
         c.nbetadt[t] = t < m.nterms ? (T)(-m.beta[t] * dt) : T(0);
     }
+    c.deg = m.rat.deg;
+    for (int i = 0; i < m.rat.deg; ++i) c.rnum[i] = (T)(-m.rat.num[i] * dt);
+    for (int i = 0; i <= m.rat.deg; ++i) c.rden[i] = (T)m.rat.den[i];
+    c.q_lo = (T)m.rat.q_lo;
     // S1 = F'_z + t, S2 = E'_z + F'_{z-1} + F'_{z+1} + 4t, S3 = E'_{z-1} + E'_{z+1} + 4t
     double ct = m.c_shell[0];
     if (stencil >= 18) ct += 4.0 * m.c_shell[1];

@@ -75,6 +75,11 @@ struct StepCoef {
     // t = (phi_{z-1} - phi) + (phi_{z+1} - phi), -beta dt, -kmu dt, -kappa dt
     T c1dt, c2dt, c3dt, ctdt, nkmudt, nkapdt;
     T nbetadt[kMaxTerms];
+    // TI: sum_k beta_k / (1 - A_k s^2) as N(q) / D(q), q = phi (1 - phi) (potential.cu):
+    // degree of D (0: none, the groups are summed one by one), coefficients of q^i in
+    // -dt N and in D, and the lowest q it covers
+    int deg;
+    T rnum[kMaxTerms], rden[kMaxTerms + 1], q_lo;
     // TI_n (local normal): per-direction c_k; the scale that turns a central
     // difference of the kernels' log-odds ln or log2((1 - phi)/phi) into the
     // gradient of psi (FP32: (lambda/4) ln 2 / (2 dx), FP64: (lambda/4) / (2 dx));
@@ -116,6 +121,20 @@ __host__ __device__ inline uint32_t sr_step_key(uint32_t seed_mix, long long ste
 __host__ __device__ inline bool is_fd_scheme(int scheme)
 {
     return scheme == SPFM_FD || scheme == SPFM_FD_H5 || scheme == SPFM_FD_HABEL;
+}
+
+// Potential of a step kernel (its KIND): 0 CF; 1..4 TI global, N / D of that many
+// groups; kKindFew + 4 and + 6 TI global, N / D of degree up to 4 or 6 in place of
+// more groups (each cell's q is compared with q_lo); kKindAny the degree read at
+// run time, or none; kKindLocal TI_n.
+constexpr int kKindFew = 4, kKindAny = 11, kKindLocal = 12;
+// of a single grid (exact: N / D covers every q)
+inline int grid_kind(int scheme, int deg, bool exact)
+{
+    if (scheme == SPFM_TI_LOCAL) return kKindLocal;
+    if (is_fd_scheme(scheme)) return 0;
+    if (deg >= 1 && deg <= 4 && exact) return deg;
+    return deg >= 1 && deg <= 4 ? kKindFew + 4 : (deg >= 1 && deg <= 6 ? kKindFew + 6 : kKindAny);
 }
 
 // Ghost mapping for one axis: at most one cell outside [0, n).  Returns the
@@ -291,7 +310,7 @@ struct BatchItem {
 // Per-dtype pieces of the persistent batch kernel (step_f32.cu / ...):
 // bytes of one device-side grid record, the work-list items of one grid, the
 // record of one grid, and the launch of one step over the whole work-list
-// (kind: 0 CF, else TI with up to 13 groups).
+// (kind: the KIND of the step kernel, the largest of the grids).
 size_t batch_grid_bytes_f32();
 size_t batch_grid_bytes_f64();
 size_t batch_grid_bytes_bf16();

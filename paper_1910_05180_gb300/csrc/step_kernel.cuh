@@ -39,6 +39,10 @@
 #pragma once
 
 #include <cuda.h>   // CUtensorMap (the map is encoded on the host, see tma.cu)
+#include <math.h>
+#include <string.h>
+
+#include <type_traits>
 
 #include "spfm_internal.h"
 
@@ -105,21 +109,51 @@ template <> struct PackT<double> { using P = D2; static P splat(double v) { retu
 
 // Step coefficients pre-splatted into packs (kernel parameter space), with dt
 // folded in: phi' = phi + c1 dt S1' + c2 dt S2' + c3 dt S3'
-//                 + q (s sum_k (-beta_k dt)/(1 - A_k s^2) - kmu dt)      (TI)
+//                 + q (s (-dt) N(q) / D(q) - kmu dt)                    (TI)
 //                 + q (s (-kappa dt) - kmu dt)                          (CF)
+// with N(q) / D(q) = sum_k beta_k / (1 - A_k s^2) (potential.cu).
 template <class T>
 struct PackCoef {
     using P = typename PackT<T>::P;
     P one, m2, m4, c1, c2, c3, ct, nkmu, nkap;
-    P nA[kMaxTerms], nbeta[kMaxTerms];   // -A_k and -beta_k dt of the coupling groups
-    int nterms;
-    // the same pairs side by side (one 16- or 32-byte load each), read by the
-    // run-time group count path, whose coefficients may sit in global memory
+    // coefficients of q^i in -dt N and in D, side by side (one 16- or 32-byte
+    // load: a batch reads them from its grid records in global memory)
+    struct __align__(2 * sizeof(P)) Ratio {
+        P num, den;
+    };
+    Ratio rat[kMaxTerms + 1];
+    int deg;          // degree of D (0: the coupling groups are summed one by one)
+    uint32_t guard;   // bits of the lowest q that N / D covers (potential.cu)
+    // -A_k and -beta_k dt of the coupling groups, for the sum group by group
     struct __align__(2 * sizeof(P)) Pair {
         P nA, nbeta;
     };
+    int nterms;
     Pair pair[kMaxTerms];
 };
+
+// the upper 32 bits of a value; for a negative limit l, bits(x) > bits(l) as
+// unsigned numbers exactly where x < l (or x is a NaN with its sign set)
+__host__ __device__ __forceinline__ uint32_t top_bits(float x)
+{
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(x);
+#else
+    uint32_t b;
+    memcpy(&b, &x, 4);
+    return b;
+#endif
+}
+__host__ __device__ __forceinline__ uint32_t top_bits(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (uint32_t)__double2hiint(x);
+#else
+    uint64_t b;
+    memcpy(&b, &x, 8);
+    return (uint32_t)(b >> 32);
+#endif
+}
 
 template <class T>
 inline PackCoef<T> make_pack_coef(const StepCoef<T> &c)
@@ -136,12 +170,16 @@ inline PackCoef<T> make_pack_coef(const StepCoef<T> &c)
     p.nkmu = PT::splat(c.nkmudt);
     p.nkap = PT::splat(c.nkapdt);
     for (int k = 0; k < kMaxTerms; ++k) {
-        p.nA[k] = PT::splat(-c.A[k]);
-        p.nbeta[k] = PT::splat(c.nbetadt[k]);
-        p.pair[k].nA = p.nA[k];
-        p.pair[k].nbeta = p.nbeta[k];
+        p.pair[k].nA = PT::splat(-c.A[k]);
+        p.pair[k].nbeta = PT::splat(c.nbetadt[k]);
     }
     p.nterms = c.nterms;
+    for (int i = 0; i <= kMaxTerms; ++i) {
+        p.rat[i].num = PT::splat(i < kMaxTerms ? c.rnum[i] : T(0));
+        p.rat[i].den = PT::splat(c.rden[i]);
+    }
+    p.deg = c.deg;
+    p.guard = top_bits(c.q_lo);
     return p;
 }
 
@@ -615,19 +653,15 @@ __device__ __forceinline__ P laplace_update(const PCoef &PC, P t, P ph, P h, P g
     return acc;
 }
 
-// KIND: 0 = CF potential; 1..4 = TI global with exactly KIND coupling groups;
-// 5 = TI global with up to 13 groups (count read at run time)
+// KIND: the potential (spfm_internal.h).  Degrees below the kernel's are padded
+// with zero coefficients, which changes no bit.
 // One tile (bx, by) of planes zc0..zc1-1.  The stage ring continues across the
 // tiles a CTA processes: plane i of this tile is ring slot base + i.  The
 // producer waits for its copies in flight before returning when drain is set.
 // Returns false when a bounded wait gave up (the error word is set).
 // SR: stochastic rounding of the update (FP32 compute only), random bits from
 // sr_hash(padded cell index xor sr_key).
-// ROLL (KIND 5): the group loop stays a loop, for coefficients in the kernel's
-// parameters (single grids); from a batch's grid records in global memory the
-// unrolled loop overlaps the pairs' loads.  Same operations, same bits.
-template <class S, class T, int STENCIL, int KIND, int TX, int TY, int RPT_, bool IMG = false, bool SR = false,
-          bool ROLL = false>
+template <class S, class T, int STENCIL, int KIND, int TX, int TY, int RPT_, bool IMG = false, bool SR = false>
 __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T> &PC,
                                           const S *__restrict__ src, S *__restrict__ dst,
                                           int *__restrict__ err, const CUtensorMap *tmap, int bx,
@@ -642,8 +676,10 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
     using P = typename K::P;
     constexpr int VX = Sh::VX, NP = Sh::NP, W = Sh::W, SW = Sh::SW, ROWS = Sh::ROWS;
     constexpr int STAGE = Sh::STAGE, NS = Sh::NS;
-    constexpr int NTMAX = KIND >= 1 && KIND <= 4 ? KIND : kMaxTerms;
-    static_assert(KIND != 6 || RPT_ == 1, "TI_n runs one row per thread");
+    constexpr bool kGlobal = KIND != 0 && KIND != kKindLocal;
+    constexpr bool kGuard = KIND > 4;                       // q below q_lo: group by group
+    constexpr int DEG = KIND > kKindFew ? KIND - kKindFew : KIND;
+    static_assert(KIND != kKindLocal || RPT_ == 1, "TI_n runs one row per thread");
 
     const GridGeom &g = C.g;
     const int tid = threadIdx.x;
@@ -811,13 +847,13 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                         p[r].g[q] = STENCIL == 26 ? K::fma(PC.c3, e, K::mul(PC.c2, f)) : f;
                     }
                 }
-                if (KIND == 6) {
+                if (KIND == kKindLocal) {
                     // log-odds at the cells and central differences along x and y.  A
                     // warp holds 32/TX rows: each lane inverts its own cells and
                     // its row's two x-neighbour cells; the rows above and below
                     // come by shuffle from the lanes TX away, except beyond the
                     // warp's first and last rows, where the lane inverts them.
-                    static_assert(KIND != 6 || (TX <= 16 && 32 % TX == 0), "TI_n needs two or more rows a warp");
+                    static_assert(KIND != kKindLocal || (TX <= 16 && 32 % TX == 0), "TI_n needs two or more rows a warp");
                     const T ep = C.eps;
                     const bool first = lane < TX, last = lane >= 32 - TX;
                     T own[VX], outer[VX];
@@ -866,46 +902,75 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                 // padded index of the row's first cell (32-bit, wraps): the cell's
                 // part of the stochastic-rounding hash
                 const uint32_t sr_row = SR ? (uint32_t)cell_index(g, gx, gy + r, oz) : 0u;
-                if constexpr (KIND == 5) {
-                    // up to 13 groups counted at run time (in a batch the coefficients
-                    // sit in global memory): the running fraction over every pack of
-                    // the row per group, so that each (A, beta) pair is read once a row
-                    P acc[NP], sg[NP], q1[NP], u[NP], num[NP], den[NP];
-                    const typename PackCoef<T>::Pair t0 = PC.pair[0];
-#pragma unroll
-                    for (int q = 0; q < NP; ++q) {
+                if constexpr (kGlobal) {
+                    // w = s (-dt) N(q) / D(q) - kmu dt by Horner's rule (2 DEG - 1 FMAs; the
+                    // running fraction it replaces took 4 operations a group: 512^3
+                    // TI_<120> 211.6 -> 194.9 us a step, 13 groups at 150 x 133 x 117
+                    // 19.6 -> 12.4, a 64-grid sweep step 156 -> 92); a thread with a cell
+                    // below the guard (or a grid without N / D) sums its coupling groups
+                    // one by one as that fraction
+                    auto pack = [&](int q, auto by_group) -> P {
                         const P ph = z[r].c[q];
                         const P t = K::add(K::sub(m[r].c[q], ph), K::sub(p[r].c[q], ph));
                         // SR: the increment alone, phi is added once in sr_update
-                        acc[q] = laplace_update<SR, STENCIL>(PC, t, ph, z[r].h[q], m[r].g[q], p[r].g[q]);
-                        sg[q] = K::fma(PC.m2, ph, PC.one);
-                        q1[q] = K::mul(ph, K::sub(PC.one, ph));
-                        u[q] = K::mul(sg[q], sg[q]);
-                        num[q] = t0.nbeta;
-                        den[q] = K::fma(t0.nA, u[q], PC.one);
-                    }
-                    auto group = [&](const typename PackCoef<T>::Pair tk) {
-#pragma unroll
-                        for (int q = 0; q < NP; ++q) {
-                            const P d = K::fma(tk.nA, u[q], PC.one);
-                            num[q] = K::fma(num[q], d, K::mul(tk.nbeta, den[q]));
-                            den[q] = K::mul(den[q], d);
-                        }
-                    };
-                    if constexpr (ROLL) {
+                        const P acc = laplace_update<SR, STENCIL>(PC, t, ph, z[r].h[q], m[r].g[q], p[r].g[q]);
+                        const P sg = K::fma(PC.m2, ph, PC.one);
+                        const P q1 = K::mul(ph, K::sub(PC.one, ph));
+                        P num, den;
+                        if constexpr (by_group.value) {
+                            const P u = K::mul(sg, sg);
+                            const typename PackCoef<T>::Pair t0 = PC.pair[0];
+                            num = t0.nbeta;
+                            den = K::fma(t0.nA, u, PC.one);
 #pragma unroll 1
-                        for (int kk = 1; kk < PC.nterms; ++kk) group(PC.pair[kk]);
-                    } else {
+                            for (int kk = 1; kk < PC.nterms; ++kk) {
+                                const typename PackCoef<T>::Pair tk = PC.pair[kk];
+                                const P d = K::fma(tk.nA, u, PC.one);
+                                num = K::fma(num, d, K::mul(tk.nbeta, den));
+                                den = K::mul(den, d);
+                            }
+                        } else if constexpr (KIND == kKindAny) {
+                            const int n = PC.deg;
+                            num = PC.rat[n - 1].num;
+                            den = K::fma(PC.rat[n].den, q1, PC.rat[n - 1].den);
+#pragma unroll 1
+                            for (int i = n - 2; i >= 0; --i) {
+                                const typename PackCoef<T>::Ratio c = PC.rat[i];
+                                num = K::fma(num, q1, c.num);
+                                den = K::fma(den, q1, c.den);
+                            }
+                        } else {
+                            num = PC.rat[DEG - 1].num;
+                            den = K::fma(PC.rat[DEG].den, q1, DEG == 1 ? PC.one : PC.rat[DEG - 1].den);
 #pragma unroll
-                        for (int kk = 1; kk < NTMAX; ++kk)
-                            if (kk < PC.nterms) group(PC.pair[kk]);
-                    }
-#pragma unroll
-                    for (int q = 0; q < NP; ++q) {
-                        P o = K::fma(q1[q], K::fma(sg[q], K::div(num[q], den[q]), PC.nkmu), acc[q]);
-                        if constexpr (SR) o = sr_update<S>(z[r].c[q], o, sr_hash((sr_row + 2 * q) ^ sr_key));
+                            for (int i = DEG - 2; i >= 0; --i) {
+                                const typename PackCoef<T>::Ratio c = PC.rat[i];
+                                num = K::fma(num, q1, c.num);
+                                den = K::fma(den, q1, i == 0 ? PC.one : c.den);
+                            }
+                        }
+                        const P w = K::fma(sg, K::div(num, den), PC.nkmu);
+                        P o = K::fma(q1, w, acc);
+                        if constexpr (SR) o = sr_update<S>(ph, o, sr_hash((sr_row + 2 * q) ^ sr_key));
                         outv[2 * q] = o.x;
                         outv[2 * q + 1] = o.y;
+                        return q1;
+                    };
+                    bool groups = KIND == kKindAny && PC.deg == 0;
+                    if (!groups) {
+                        uint32_t low = 0u;
+#pragma unroll
+                        for (int q = 0; q < NP; ++q) {
+                            const P q1 = pack(q, std::false_type{});
+                            if constexpr (kGuard) low = max(low, max(top_bits(q1.x), top_bits(q1.y)));
+                        }
+                        if constexpr (kGuard) groups = low > PC.guard;
+                    }
+                    if constexpr (kGuard) {
+                        if (groups) {
+#pragma unroll
+                            for (int q = 0; q < NP; ++q) pack(q, std::true_type{});
+                        }
                     }
                 } else {
 #pragma unroll
@@ -928,23 +993,11 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                                 drive = K::div(PC.nkmu, K::mul(K::mk(T(3), T(3)), K::mul(d, d)));
                             }
                             w = K::fma(sg, PC.nkap, drive);
-                        } else if (KIND == 6) {
+                        } else {
                             const P s2 = K::mk(C.psi_grad, C.psi_grad);
                             const P gz = K::mul(K::sub(p[r].psi[q], m[r].psi[q]), s2);
                             w = ti_local_w<T, STENCIL>(C, sg, K::mul(sg, sg), K::mul(z[r].gx[q], s2),
                                                        K::mul(z[r].gy[q], s2), gz);
-                        } else {
-                            // exactly KIND groups, coefficients from the parameter bank
-                            const P u = K::mul(sg, sg);
-                            P num = PC.nbeta[0];
-                            P den = K::fma(PC.nA[0], u, PC.one);
-#pragma unroll
-                            for (int kk = 1; kk < NTMAX; ++kk) {
-                                const P d = K::fma(PC.nA[kk], u, PC.one);
-                                num = K::fma(num, d, K::mul(PC.nbeta[kk], den));
-                                den = K::mul(den, d);
-                            }
-                            w = K::fma(sg, K::div(num, den), PC.nkmu);
                         }
                         P o = K::fma(q1, w, acc);
                         if constexpr (SR) o = sr_update<S>(ph, o, sr_hash((sr_row + 2 * q) ^ sr_key));
@@ -1006,12 +1059,13 @@ template <class S> struct MinBlocks { static constexpr int value = SPFM_MIN_CTAS
 template <> struct MinBlocks<float> { static constexpr int value = 4; };
 template <class S> struct BatchMinBlocks { static constexpr int value = SPFM_MIN_CTAS; };
 
-// (the stochastic-rounding kernels and the 13-group potential keep three CTAs
-// per SM: at four their registers spill, and the 13-group kernel ran 15-18 %
-// slower at 192^3)
+// (the stochastic-rounding kernels and the potentials with the guard on q keep
+// three CTAs per SM: at four their registers spill; 150 x 133 x 117 with a
+// random normal 12.4 us a step at three, 12.6 at four, and the guard in the
+// kernels of 1 to 4 groups, which do not need it, cost 18 % at 512^3)
 template <class S, class T, int STENCIL, int KIND, int TX, int TY, int RPT_, bool IMG, bool SR = false>
 __global__ void __launch_bounds__(TileShape<S, T, TX, TY, RPT_>::NTHREADS,
-                                  RPT_ == 1 ? 2 : ((SR || KIND == 5) ? SPFM_MIN_CTAS : MinBlocks<S>::value))
+                                  RPT_ == 1 ? 2 : ((SR || KIND > 4) ? SPFM_MIN_CTAS : MinBlocks<S>::value))
     spfm_step_kernel(const StepCoef<T> C, const PackCoef<T> PC, const S *__restrict__ src,
                      S *__restrict__ dst, int *__restrict__ err, int zchunk,
                      const __grid_constant__ CUtensorMap tmap, int use_tmap, int mode)
@@ -1041,7 +1095,7 @@ __global__ void __launch_bounds__(TileShape<S, T, TX, TY, RPT_>::NTHREADS,
 #pragma unroll
         for (int f = 0; f < 6; ++f) fwd = fwd && C.g.bc[f] != SPFM_PERIODIC;
     }
-    step_tile<S, T, STENCIL, KIND, TX, TY, RPT_, IMG, SR, true>(C, PC, src, dst, err, use_tmap ? &tmap : nullptr,
+    step_tile<S, T, STENCIL, KIND, TX, TY, RPT_, IMG, SR>(C, PC, src, dst, err, use_tmap ? &tmap : nullptr,
                                                      blockIdx.x, blockIdx.y, zc0, zc1, stages, full, empty, 0,
                                                      true, mode, C.sr_key, ready, fwd);
 }
@@ -1139,7 +1193,9 @@ cudaError_t launch_batch_t(const void *grids, const BatchItem *work, int nwork, 
 #define SPFM_BBY_KIND(ST)                      \
     do {                                       \
         if (kind == 0) SPFM_BLAUNCH(ST, 0);    \
-        else SPFM_BLAUNCH(ST, 5);              \
+        else if (kind <= kKindFew + 4) SPFM_BLAUNCH(ST, kKindFew + 4); \
+        else if (kind <= kKindFew + 6) SPFM_BLAUNCH(ST, kKindFew + 6); \
+        else SPFM_BLAUNCH(ST, kKindAny);       \
     } while (0)
     if (stencil == 6) SPFM_BBY_KIND(6);
     else if (stencil == 18) SPFM_BBY_KIND(18);
@@ -1160,11 +1216,7 @@ cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int target = 6 * MinBlocks<S>::value * sms;
-    // exact group counts 1..4 get their own kernels; 0 groups (all A_k = 0)
-    // runs the one-group kernel with beta = 0
-    const int kind = is_fd_scheme(cfg.scheme) ? 0
-                     : cfg.scheme == SPFM_TI_LOCAL ? 6
-                                                   : (c.nterms <= 4 ? (c.nterms < 1 ? 1 : c.nterms) : 5);
+    const int kind = grid_kind(cfg.scheme, c.deg, isinf(c.q_lo));
     const PackCoef<T> pc = make_pack_coef<T>(c);
     CUtensorMap map;
     if (tmap) map = *tmap;
@@ -1203,8 +1255,10 @@ cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, 
         else if (kind == 2) SPFM_LAUNCH(ST, 2); \
         else if (kind == 3) SPFM_LAUNCH(ST, 3); \
         else if (kind == 4) SPFM_LAUNCH(ST, 4); \
-        else if (kind == 5) SPFM_LAUNCH(ST, 5); \
-        else le = go(spfm_step_kernel<S, T, ST, 6, TX, TY, 1, IMG, SR>, NT1); \
+        else if (kind == kKindFew + 4) SPFM_LAUNCH(ST, kKindFew + 4); \
+        else if (kind == kKindFew + 6) SPFM_LAUNCH(ST, kKindFew + 6); \
+        else if (kind == kKindAny) SPFM_LAUNCH(ST, kKindAny); \
+        else le = go(spfm_step_kernel<S, T, ST, kKindLocal, TX, TY, 1, IMG, SR>, NT1); \
     } while (0)
     if (cfg.stencil == 6) SPFM_BY_KIND(6);
     else if (cfg.stencil == 18) SPFM_BY_KIND(18);
