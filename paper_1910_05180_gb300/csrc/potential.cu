@@ -14,8 +14,8 @@
 // with it in 2 N points of [0, u_hi] comes from the Gauss quadrature of the
 // measure beta_k / prod_i (1 - u_i A_k) (multipoint Pade approximation of
 // Stieltjes functions; see Stahl and Totik, "General Orthogonal Polynomials",
-// 1992, ch. 6), here by Lanczos' algorithm on the K masses and Jacobi
-// rotations (Golub and Welsch, Math. Comp. 23, 1969).  The nodes stay inside
+// 1992, ch. 6), here by Lanczos' algorithm on the K masses and QL
+// iterations (Golub and Welsch, Math. Comp. 23, 1969).  The nodes stay inside
 // the range of the A_k and the weights stay positive, so the form above is
 // kept.  The u_i are Chebyshev points in log(1 / A_max - u), which crowds them
 // where the nearest pole is felt: the error falls below 2^-30 of the sum with
@@ -38,51 +38,51 @@ constexpr int kK = spfm::kMaxTerms;
 constexpr double kTol = 0x1p-30;
 constexpr double kMaxCoef = 1e24;   // FP32 range of the coefficients, with room for q outside [0, 1/4]
 
-// eigenvalues of the symmetric n x n matrix a and the first components of its
-// eigenvectors, by cyclic Jacobi rotations
-void jacobi(double a[kK][kK], int n, double *x, double *v0)
+// Eigenvalues d and first components z of the unit eigenvectors of the n x n
+// symmetric tridiagonal matrix with diagonal d and off-diagonal e, by QL
+// iterations with Wilkinson's shift (Golub and Welsch); false without convergence.
+bool eigen(double *d, double *e, double *z, int n)
 {
-    double v[kK][kK];
-    for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) v[i][j] = i == j ? 1.0 : 0.0;
-    for (int sweep = 0; sweep < 30; ++sweep) {
-        double off = 0.0, diag = 0.0;
-        for (int i = 0; i < n; ++i) {
-            diag += a[i][i] * a[i][i];
-            for (int j = 0; j < i; ++j) off += a[i][j] * a[i][j];
-        }
-        if (off <= 1e-34 * diag) break;
-        for (int p = 0; p < n - 1; ++p)
-            for (int q = p + 1; q < n; ++q) {
-                if (a[p][q] == 0.0) continue;
-                const double th = (a[q][q] - a[p][p]) / (2.0 * a[p][q]);
-                const double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-                const double c = 1.0 / sqrt(t * t + 1.0), s = t * c;
-                for (int k = 0; k < n; ++k) {
-                    const double kp = a[k][p], kq = a[k][q];
-                    a[k][p] = c * kp - s * kq;
-                    a[k][q] = s * kp + c * kq;
-                }
-                for (int k = 0; k < n; ++k) {
-                    const double pk = a[p][k], qk = a[q][k], vp = v[k][p], vq = v[k][q];
-                    a[p][k] = c * pk - s * qk;
-                    a[q][k] = s * pk + c * qk;
-                    v[k][p] = c * vp - s * vq;
-                    v[k][q] = s * vp + c * vq;
+    for (int i = 0; i < n; ++i) z[i] = i == 0 ? 1.0 : 0.0;
+    e[n - 1] = 0.0;
+    for (int l = 0; l < n; ++l)
+        for (int it = 0;; ++it) {
+            int m = l;   // the block l..m is unreduced
+            while (m < n - 1 && fabs(e[m]) > 1e-17 * (fabs(d[m]) + fabs(d[m + 1]))) ++m;
+            if (m == l) break;
+            if (it == 50) return false;
+            // the shift: the eigenvalue of the leading 2 x 2 block nearer d[l]
+            const double h = (d[l + 1] - d[l]) / (2.0 * e[l]);
+            const double shift = d[l] - e[l] / (h + copysign(sqrt(h * h + 1.0), h));
+            // one sweep of plane rotations from the bottom chases the bulge up
+            double x = d[m] - shift, y = e[m - 1];
+            for (int i = m - 1; i >= l; --i) {
+                const double r = sqrt(x * x + y * y);
+                if (r == 0.0) break;
+                const double c = x / r, s = y / r;   // rotates (i, i + 1)
+                if (i < m - 1) e[i + 1] = r;
+                const double a = d[i], b = e[i], f = d[i + 1];
+                d[i + 1] = c * c * f + 2.0 * c * s * b + s * s * a;
+                d[i] = s * s * f - 2.0 * c * s * b + c * c * a;
+                e[i] = c * s * (a - f) + (c * c - s * s) * b;
+                const double t = z[i + 1];
+                z[i + 1] = c * t + s * z[i];
+                z[i] = c * z[i] - s * t;
+                if (i > l) {
+                    x = e[i];
+                    y = s * e[i - 1];
+                    e[i - 1] *= c;
                 }
             }
-    }
-    for (int i = 0; i < n; ++i) {
-        x[i] = a[i][i];
-        v0[i] = v[0][i];
-    }
+        }
+    return true;
 }
 
 // N nodes and weights whose sum of w / (1 - x u) agrees with that of
 // (A, beta) in the 2 N points u
 bool reduce(const double *A, const double *beta, int K, int N, const double *u, double *x, double *w)
 {
-    double Q[kK][kK], T[kK][kK], total = 0.0;
+    double Q[kK][kK], off[kK], v0[kK], total = 0.0;
     for (int k = 0; k < K; ++k) {
         double om = 1.0;
         for (int i = 0; i < 2 * N; ++i) om *= 1.0 - u[i] * A[k];
@@ -90,12 +90,10 @@ bool reduce(const double *A, const double *beta, int K, int N, const double *u, 
         total += Q[0][k];
     }
     for (int k = 0; k < K; ++k) Q[0][k] = sqrt(Q[0][k] / total);
-    for (int i = 0; i < N; ++i)
-        for (int j = 0; j < N; ++j) T[i][j] = 0.0;
     for (int n = 0; n < N; ++n) {
         double a = 0.0, r[kK], norm = 0.0;
         for (int k = 0; k < K; ++k) a += A[k] * Q[n][k] * Q[n][k];
-        T[n][n] = a;
+        x[n] = a;
         if (n == N - 1) break;
         for (int k = 0; k < K; ++k) r[k] = A[k] * Q[n][k];
         for (int pass = 0; pass < 2; ++pass)   // orthogonal to all before, twice
@@ -107,11 +105,10 @@ bool reduce(const double *A, const double *beta, int K, int N, const double *u, 
         for (int k = 0; k < K; ++k) norm += r[k] * r[k];
         norm = sqrt(norm);
         if (!(norm > 1e-14 * a)) return false;   // fewer than N distinct masses
-        T[n][n + 1] = T[n + 1][n] = norm;
+        off[n] = norm;
         for (int k = 0; k < K; ++k) Q[n + 1][k] = r[k] / norm;
     }
-    double v0[kK];
-    jacobi(T, N, x, v0);
+    if (!eigen(x, off, v0, N)) return false;
     for (int j = 0; j < N; ++j) {
         double om = total * v0[j] * v0[j];
         for (int i = 0; i < 2 * N; ++i) om *= 1.0 - u[i] * x[j];
@@ -154,7 +151,8 @@ void build_rational(const double *A, const double *E, const double *beta, int K,
         for (int k = 0; k < K; ++k) amax = std::max(amax, A[k]);
         const double pole = 1.0 / amax, u_hi = 1.0 + std::min(0.05, 0.25 * (pole - 1.0));
         const double l0 = log(pole), l1 = log(pole - u_hi);
-        for (int N = 2; N < K && pole - u_hi > 0.0; ++N) {
+        // a generic normal needs about 2.7 + log(pole / (pole - u_hi)) terms: the search starts there
+        for (int N = std::max(2, (int)(2.7 + l0 - l1)); N < K && pole - u_hi > 0.0; ++N) {
             double u[2 * kK], x[kK], w[kK], e[kK];
             for (int i = 0; i < 2 * N; ++i)
                 u[i] = pole - exp(l0 + (l1 - l0) * 0.5 * (1.0 - cos(M_PI * (2 * i + 1) / (4.0 * N))));
