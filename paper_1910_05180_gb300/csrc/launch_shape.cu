@@ -23,8 +23,17 @@
 //   where chunks of 16 planes or more lost up to 2x on grids of 96^3 ... 192^3.
 //   The model takes a CTA's speed as independent of the CTAs beside it on its
 //   SM, which holds for the streaming kernels at three or four CTAs per SM;
-//   kernels with fewer (TI_n: two, bound by instruction issue, where a CTA
-//   left alone on an SM runs faster) keep the rule of many rounds.
+//   kernels with fewer keep the rule of many rounds.
+//
+// TI_n has a rule of its own: its CTAs differ in work (those in the interface
+// band compute the 13 couplings of each cell, a plane of them some 2 us; those
+// in the bulk do not), so it wants many small CTAs.  About six rounds of
+// the slots, chunks of 4 to 16 planes; where chunks of 4 leave slots empty, the
+// shortest chunks that still fit one round.  Measured at two CTAs per SM (us a
+// step, FP32 27-point, planes per CTA): 60^3 cube 20: 37.9, 4: 12.6, 1 (chosen):
+// 10.1; 64^3 plane all in the band 16: 40.0, 4: 13.8, 1 (chosen): 7.4; 96^3 16:
+// 46.2, 4 (chosen): 15.5, 2: 16.3; 192^3 16: 72, 4 (chosen): 60.5, 2: 69.8;
+// 256^3 16: 96.0, 8: 90.4 (9 chosen), 4: 94.2; 320^3 16 (chosen): 124.6, 8: 129.
 #include <map>
 #include <mutex>
 #include <queue>
@@ -87,14 +96,25 @@ static int model_zchunk(int tiles, int nz, int per_sm, int slots, int target)
     return best;
 }
 
+// planes per CTA of a TI_n launch (see above)
+static int uneven_zchunk(int tiles, int nz, int slots)
+{
+    if ((long long)tiles * ((nz + 3) / 4) < slots) {
+        const int chunks = slots / tiles < nz ? slots / tiles : nz;
+        return (nz + chunks - 1) / chunks;
+    }
+    const long long zc = ((long long)tiles * nz + 6LL * slots - 1) / (6LL * slots);
+    return zc < 4 ? 4 : (zc > 16 ? 16 : (int)zc);
+}
+
 namespace {
 std::mutex g_mu;
-// (kernel, threads, device) -> resident CTAs per SM; (tiles, nz, slots, target) -> z-chunk
+// (kernel, threads, device) -> resident CTAs per SM; (tiles, nz, slots, target or -1: uneven) -> z-chunk
 std::map<std::tuple<const void *, int, int>, int> g_occ;
 std::map<std::tuple<int, int, int, int>, int> g_zc;
 }  // namespace
 
-int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target)
+int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target, bool uneven)
 {
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
@@ -114,11 +134,11 @@ int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target)
         g_occ[ok] = per_sm;
     }
     const int slots = per_sm * sms;
-    const auto zk = std::make_tuple(tiles, nz, slots, target);
+    const auto zk = std::make_tuple(tiles, nz, slots, uneven ? -1 : target);
     auto z = g_zc.find(zk);
     if (z != g_zc.end()) return z->second;
     if (g_zc.size() >= 4096) g_zc.clear();   // many grid shapes (a serving process): start over
-    const int zc = model_zchunk(tiles, nz, per_sm, slots, target);
+    const int zc = uneven ? uneven_zchunk(tiles, nz, slots) : model_zchunk(tiles, nz, per_sm, slots, target);
     g_zc[zk] = zc;
     return zc;
 }

@@ -356,30 +356,53 @@ template <class T, int NP>
 struct PlaneQ {
     using P = typename Pk<T>::P;
     P c[NP], h[NP], g[NP];
-    P psi[NP], gx[NP], gy[NP];   // TI_n only: log-odds of phi and its in-plane differences
+    // TI_n only: 1 or 2 where phi is at or beyond the lower or upper clamp of the
+    // profile inversion, else 0: at the row's own cells (own), and at those and
+    // their in-plane face neighbours (level)
+    int own, level;
 };
 
 // ----------------------------------------------------------------- TI_n
 
 // Inversion of the ideal profile, psi = (lambda/2) artanh(1 - 2 phi)
 // = (lambda/4) ln((1 - phi)/phi), with phi clamped to [eps, 1 - eps] (TI_n).
-// The kernels keep the log-odds only (FP32 log2, FP64 ln) and scale their
-// central differences by StepCoef::psi_grad; the FP32 log-odds is the
-// hardware log2 itself, no product, so differences of equal values are 0.
-__device__ __forceinline__ float log_odds(float phi, float eps)
+// Only its differences are needed: log-odds(a) - log-odds(b)
+// = log((1 - a) b / (a (1 - b))), FP32 in log2 as the difference of the two
+// products' logarithms, FP64 the natural logarithm of their quotient; the
+// kernels scale it by StepCoef::psi_grad.  For a = b the products are the same
+// number, so the difference is exactly zero (a clamped region keeps the CF
+// fallback).
+__device__ __forceinline__ float2 clamp_pack(float2 v, float eps)
 {
-    const float pc = fminf(fmaxf(phi, eps), 1.0f - eps);
-    return __log2f(__fdividef(1.0f - pc, pc));
+    return make_float2(fminf(fmaxf(v.x, eps), 1.0f - eps), fminf(fmaxf(v.y, eps), 1.0f - eps));
 }
-__device__ __forceinline__ double log_odds(double phi, double eps)
+__device__ __forceinline__ D2 clamp_pack(D2 v, double eps)
 {
-    const double pc = fmin(fmax(phi, eps), 1.0 - eps);
-    return log((1.0 - pc) / pc);
+    return {fmin(fmax(v.x, eps), 1.0 - eps), fmin(fmax(v.y, eps), 1.0 - eps)};
 }
-template <class T>
-__device__ __forceinline__ typename Pk<T>::P log_odds_pack(typename Pk<T>::P v, T eps)
+__device__ __forceinline__ float2 log_ratio(float2 n, float2 d)
 {
-    return Pk<T>::mk(log_odds(v.x, eps), log_odds(v.y, eps));
+    return make_float2(__log2f(n.x) - __log2f(d.x), __log2f(n.y) - __log2f(d.y));
+}
+__device__ __forceinline__ D2 log_ratio(D2 n, D2 d) { return {log(n.x / d.x), log(n.y / d.y)}; }
+// a and b clamped; na = 1 - a, nb = 1 - b
+template <class P>
+__device__ __forceinline__ P log_odds_diff(P a, P na, P b, P nb)
+{
+    using K = Pk<decltype(P().x)>;
+    return log_ratio(K::mul(na, b), K::mul(a, nb));
+}
+// phi at or beyond the clamp, for a set of cells given by the largest and
+// smallest of their upper 32 bits as signed integers: 1 all at or below eps, 2
+// all at or above 1 - eps, else 0 (FP64 compares the upper words, which at a
+// limit's own upper word says 0: such cells take the general form, as they may)
+__device__ __forceinline__ int clamp_level(int hi, int lo, float eps)
+{
+    return hi <= __float_as_int(eps) ? 1 : (lo >= __float_as_int(1.0f - eps) ? 2 : 0);
+}
+__device__ __forceinline__ int clamp_level(int hi, int lo, double eps)
+{
+    return hi < __double2hiint(eps) ? 1 : (lo > __double2hiint(1.0 - eps) ? 2 : 0);
 }
 // tanh of a pack.  FP32: Lambert's continued fraction for tanh truncated
 // after the term x^2/11, x (10395 + 1260 y + 21 y^2) / (10395 + 4725 y + 210 y^2 + y^3)
@@ -679,7 +702,6 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
     constexpr bool kGlobal = KIND != 0 && KIND != kKindLocal;
     constexpr bool kGuard = KIND > 4;                       // q below q_lo: group by group
     constexpr int DEG = KIND > kKindFew ? KIND - kKindFew : KIND;
-    static_assert(KIND != kKindLocal || RPT_ == 1, "TI_n runs one row per thread");
 
     const GridGeom &g = C.g;
     const int tid = threadIdx.x;
@@ -825,8 +847,31 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
             P rc[RPT + 2][NP], rw[RPT + 2][NP], re[RPT + 2][NP];
 #pragma unroll
             for (int r = 0; r < RPT + 2; ++r) get_row<S, T, VX>(r0 + r * SW, rc[r], rw[r], re[r]);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[s]);
+            // TI_n reads the plane's neighbours again when it is the centre plane, and
+            // releases it then
+            if constexpr (KIND != kKindLocal) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&empty[s]);
+            } else {
+                int hi[RPT + 2], lo[RPT + 2];
+#pragma unroll
+                for (int r = 0; r < RPT + 2; ++r) {
+                    hi[r] = lo[r] = (int)top_bits(rc[r][0].x);
+#pragma unroll
+                    for (int e = 1; e < VX; ++e) {
+                        const int b = (int)top_bits(e & 1 ? rc[r][e / 2].y : rc[r][e / 2].x);
+                        hi[r] = max(hi[r], b);
+                        lo[r] = min(lo[r], b);
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < RPT; ++r) {
+                    const int w = (int)top_bits(rw[r + 1][0].x), e = (int)top_bits(re[r + 1][NP - 1].y);
+                    p[r].own = clamp_level(hi[r + 1], lo[r + 1], C.eps);
+                    p[r].level = clamp_level(max(max(max(hi[r], hi[r + 1]), hi[r + 2]), max(w, e)),
+                                             min(min(min(lo[r], lo[r + 1]), lo[r + 2]), min(w, e)), C.eps);
+                }
+            }
 #pragma unroll
             for (int r = 0; r < RPT; ++r) {
 #pragma unroll
@@ -845,50 +890,6 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                                                             K::add(rw[r + 2][q], re[r + 2][q])));
                         p[r].h[q] = K::fma(PC.c2, e, K::mul(PC.c1, f));
                         p[r].g[q] = STENCIL == 26 ? K::fma(PC.c3, e, K::mul(PC.c2, f)) : f;
-                    }
-                }
-                if (KIND == kKindLocal) {
-                    // log-odds at the cells and central differences along x and y.  A
-                    // warp holds 32/TX rows: each lane inverts its own cells and
-                    // its row's two x-neighbour cells; the rows above and below
-                    // come by shuffle from the lanes TX away, except beyond the
-                    // warp's first and last rows, where the lane inverts them.
-                    static_assert(KIND != kKindLocal || (TX <= 16 && 32 % TX == 0), "TI_n needs two or more rows a warp");
-                    const T ep = C.eps;
-                    const bool first = lane < TX, last = lane >= 32 - TX;
-                    T own[VX], outer[VX];
-#pragma unroll
-                    for (int q = 0; q < NP; ++q) {
-                        const P po = log_odds_pack<T>(rc[r + 1][q], ep);
-                        const P pb = log_odds_pack<T>(first ? rc[r][q] : rc[r + 2][q], ep);
-                        p[r].psi[q] = po;
-                        own[2 * q] = po.x;
-                        own[2 * q + 1] = po.y;
-                        outer[2 * q] = pb.x;
-                        outer[2 * q + 1] = pb.y;
-                    }
-                    // the two x-neighbour cells of the thread's run
-                    const P pwe = log_odds_pack<T>(K::mk(rw[r + 1][0].x, re[r + 1][NP - 1].y), ep);
-                    const T pw = pwe.x;   // x - 1
-                    const T pe = pwe.y;   // x + VX
-#pragma unroll
-                    for (int q = 0; q < NP; ++q) {
-                        const T w0 = 2 * q == 0 ? pw : own[2 * q - 1];
-                        const T e1 = 2 * q + 2 == VX ? pe : own[2 * q + 2];
-                        // the log-odds are no products, so equal values differ by exactly
-                        // zero and a clamped region keeps the CF fallback (a difference
-                        // fused with a multiply would leave that product's rounding
-                        // error, enough to pass |g| >= 1e-8 in FP32 with a meaningless normal)
-                        p[r].gx[q] = K::sub(K::mk(own[2 * q + 1], e1), K::mk(w0, own[2 * q]));
-                        T nb[2], sb[2];
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const T up = __shfl_up_sync(0xffffffffu, own[2 * q + h], TX);
-                            const T dn = __shfl_down_sync(0xffffffffu, own[2 * q + h], TX);
-                            nb[h] = first ? outer[2 * q + h] : up;   // row j - 1
-                            sb[h] = last ? outer[2 * q + h] : dn;    // row j + 1
-                        }
-                        p[r].gy[q] = K::sub(K::mk(sb[0], sb[1]), K::mk(nb[0], nb[1]));   // psi(j + 1) - psi(j - 1)
                     }
                 }
             }
@@ -973,6 +974,43 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                         }
                     }
                 } else {
+                    P wl[NP];   // TI_n: w of the row
+                    if constexpr (KIND == kKindLocal) {
+                        // Where every face neighbour sits in the same clamp the gradient is
+                        // zero and ti_local_w falls back to the CF potential: the bulk
+                        // phases take that alone.  Elsewhere the in-plane neighbours are
+                        // read again from the centre plane's stage, which keeps the
+                        // profile inversion out of the plane records.  320^3 grain:
+                        // 258 -> 125 us a step (at two rows a thread and half the warps
+                        // 200: a CTA's planes wait for the warps inside the band).
+                        const bool bulk = z[r].level != 0 && m[r].own == z[r].level && p[r].own == z[r].level;
+                        if (bulk) {
+#pragma unroll
+                            for (int q = 0; q < NP; ++q)
+                                wl[q] = K::fma(K::fma(PC.m2, z[r].c[q], PC.one),
+                                               K::mk(-C.dt * C.kappa, -C.dt * C.kappa),
+                                               K::mk(-C.dt * C.kmu, -C.dt * C.kmu));
+                        } else {
+                            const S *row = rbase + ((I + NS - 1) % NS) * STAGE + r * SW;
+                            P c[NP], w[NP], e[NP], u[NP], v[NP], d[NP];
+                            get_row<S, T, VX>(row, c, w, e);
+                            get_row<S, T, VX>(row - SW, u, d, d);
+                            get_row<S, T, VX>(row + SW, v, d, d);
+                            const T ep = C.eps;
+                            const P s2 = K::mk(C.psi_grad, C.psi_grad);
+                            auto diff = [&](P a, P b) {
+                                a = clamp_pack(a, ep);
+                                b = clamp_pack(b, ep);
+                                return K::mul(log_odds_diff(a, K::sub(PC.one, a), b, K::sub(PC.one, b)), s2);
+                            };
+#pragma unroll
+                            for (int q = 0; q < NP; ++q) {
+                                const P sg = K::fma(PC.m2, z[r].c[q], PC.one);
+                                wl[q] = ti_local_w<T, STENCIL>(C, sg, K::mul(sg, sg), diff(e[q], w[q]),
+                                                               diff(v[q], u[q]), diff(p[r].c[q], m[r].c[q]));
+                            }
+                        }
+                    }
 #pragma unroll
                     for (int q = 0; q < NP; ++q) {
                         const P ph = z[r].c[q];
@@ -994,10 +1032,7 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                             }
                             w = K::fma(sg, PC.nkap, drive);
                         } else {
-                            const P s2 = K::mk(C.psi_grad, C.psi_grad);
-                            const P gz = K::mul(K::sub(p[r].psi[q], m[r].psi[q]), s2);
-                            w = ti_local_w<T, STENCIL>(C, sg, K::mul(sg, sg), K::mul(z[r].gx[q], s2),
-                                                       K::mul(z[r].gy[q], s2), gz);
+                            w = wl[q];
                         }
                         P o = K::fma(q1, w, acc);
                         if constexpr (SR) o = sr_update<S>(ph, o, sr_hash((sr_row + 2 * q) ^ sr_key));
@@ -1021,6 +1056,12 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                     for (int e = 0; e < VX; ++e)
                         if (gx + e < g.nx) optr[e] = Io<S, T>::cvt_out(outv[e]);
                 }
+            }
+        }
+        if constexpr (KIND == kKindLocal) {
+            if (i >= 1) {   // the plane before this one has been the centre plane
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&empty[(I + NS - 1) % NS]);
             }
         }
         return i + 1 < nplanes;
@@ -1065,7 +1106,7 @@ template <class S> struct BatchMinBlocks { static constexpr int value = SPFM_MIN
 // kernels of 1 to 4 groups, which do not need it, cost 18 % at 512^3)
 template <class S, class T, int STENCIL, int KIND, int TX, int TY, int RPT_, bool IMG, bool SR = false>
 __global__ void __launch_bounds__(TileShape<S, T, TX, TY, RPT_>::NTHREADS,
-                                  RPT_ == 1 ? 2 : ((SR || KIND > 4) ? SPFM_MIN_CTAS : MinBlocks<S>::value))
+                                  KIND == kKindLocal ? 2 : ((SR || KIND > 4) ? SPFM_MIN_CTAS : MinBlocks<S>::value))
     spfm_step_kernel(const StepCoef<T> C, const PackCoef<T> PC, const S *__restrict__ src,
                      S *__restrict__ dst, int *__restrict__ err, int zchunk,
                      const __grid_constant__ CUtensorMap tmap, int use_tmap, int mode)
@@ -1238,7 +1279,9 @@ cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, 
     // z-chunk: the caller's, else the launch-shape model's for this kernel (a
     // grid dimension stays below 65536 chunks)
     auto go = [&](auto kern, int threads) {
-        int zchunk = cfg.zchunk > 0 ? cfg.zchunk : pick_zchunk((const void *)kern, threads, gxn * gyn, c.g.nz, target);
+        int zchunk = cfg.zchunk > 0 ? cfg.zchunk
+                                    : pick_zchunk((const void *)kern, threads, gxn * gyn, c.g.nz, target,
+                                                  kind == kKindLocal);
         if (zchunk > c.g.nz) zchunk = c.g.nz;
         if (zchunk < (c.g.nz + 65534) / 65535) zchunk = (c.g.nz + 65534) / 65535;
         if (cfg.zchunk_used) *cfg.zchunk_used = zchunk;
