@@ -603,7 +603,7 @@ spfm_status spfm_step_conserving(spfm_grid *g, int n_steps, double M, double Gam
     }
     for (int i = 0; i < n_steps; ++i) {
         void *src = g->d.field[g->cur], *dst = g->d.field[1 - g->cur];
-        cfg.mode = i == 0 ? kWaitAll : kWaitFaces;   // the face kernel follows the correction
+        cfg.mode = kWaitAll | kEarly;   // the sums and the correction wait for their predecessor, too
         cf.sr_key = sr_step_key(g->sr_seed, g->steps + i);
         cudaError_t e;
         if (g->d.dtype == SPFM_F64)
@@ -613,8 +613,7 @@ spfm_status spfm_step_conserving(spfm_grid *g, int n_steps, double M, double Gam
         else
             e = launch_step_bf16(cf, (const __nv_bfloat16 *)src, (__nv_bfloat16 *)dst, err, cfg, &g->tma,
                                  g->cur, s);
-        if (e == cudaSuccess) e = launch_conserve(g->geom, g->d.dtype, src, dst, partials, alpha, s);
-        if (e == cudaSuccess) e = launch_fill_ghosts(g->geom, g->d.dtype, m.aface, dst, s, 1);
+        if (e == cudaSuccess) e = launch_conserve(g->geom, g->d.dtype, m.aface, src, dst, partials, alpha, s);
         if (e != cudaSuccess) return cuda_fail(g, e, "spfm_step_conserving");
         g->cur ^= 1;
     }

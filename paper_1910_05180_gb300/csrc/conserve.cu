@@ -8,125 +8,304 @@
 // cell with
 //     alpha = sum_p (phi*_p - phi_p) / sum_p q(phi_p),
 //     dF    = alpha lambda Gamma / (4 M dt).
-// Pass 1 reduces the two sums in FP64 (rows dealt round-robin to the blocks,
-// fixed order, so the result is reproducible); pass 2 has every block add the
-// partials in the same order, form alpha, and correct its rows of phi*.
+// Pass 1 reduces the two sums (rows dealt round-robin to the warps, fixed order,
+// so the result is reproducible); in pass 2 every block adds the partials in
+// the same order, forms alpha, corrects its rows of phi* and writes the ghost
+// cells whose source they hold, so that no face kernel follows.
+//
+// Both are bound by the FP64 pipe (a warp's FP64 instruction holds it 16 cycles
+// for the whole SM) and by latency at the grids of this study (60^3: 0.9 MB a
+// field).  So a warp takes a row in 16-byte loads; cells of FP32 and BF16 fields
+// are summed by fours and corrected in double-float pairs, whose terms are exact
+// (48 bits against the 24 of a cell), and only the sums of four enter FP64; the
+// block reduction adds 8 values a lane from shared memory before it shuffles.
+// The kernels of a step chain by programmatic dependent launch.  60^3 FP32, us
+// a step: sums 10.9 -> 6.0, correction and ghosts 67.1 + 3.4 -> 6.9 (one thread
+// added the 608 partials one by one); alpha formed once, by the last block of
+// the sums, was slower (9.1 + 5.1).
+#include "double_float.cuh"
 #include "spfm_internal.h"
 
 namespace spfm {
 
 namespace {
 
-template <class S> __device__ __forceinline__ double ld64(const S *f, long long i);
-template <> __device__ __forceinline__ double ld64<double>(const double *f, long long i) { return f[i]; }
-template <> __device__ __forceinline__ double ld64<float>(const float *f, long long i) { return (double)f[i]; }
-template <> __device__ __forceinline__ double ld64<__nv_bfloat16>(const __nv_bfloat16 *f, long long i)
+// storage <-> compute (FP64, or FP32 for FP32 and BF16 storage)
+template <class S> struct Cell {
+    using T = float;
+};
+template <> struct Cell<double> {
+    using T = double;
+};
+__device__ __forceinline__ double get(double v) { return v; }
+__device__ __forceinline__ float get(float v) { return v; }
+__device__ __forceinline__ float get(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ void put(double &s, double v) { s = v; }
+__device__ __forceinline__ void put(float &s, float v) { s = v; }
+__device__ __forceinline__ void put(__nv_bfloat16 &s, float v) { s = __float2bfloat16_rn(v); }
+
+// d - x and q(x) = x (1 - x) of the first n of a group of cells, added to the FP64 sums
+__device__ __forceinline__ void add_cells(const double *x, const double *d, int n, double &dsum, double &qsum)
 {
-    return (double)__bfloat162float(f[i]);
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+        if (e < n) {
+            dsum += d[e] - x[e];
+            qsum += fma(-x[e], x[e], x[e]);
+        }
 }
-template <class S> __device__ __forceinline__ S st_of(double v);
-template <> __device__ __forceinline__ double st_of<double>(double v) { return v; }
-template <> __device__ __forceinline__ float st_of<float>(double v) { return (float)v; }
-template <> __device__ __forceinline__ __nv_bfloat16 st_of<__nv_bfloat16>(double v)
+__device__ __forceinline__ DF q_of(float x) { return df_mul_f(df_two_sum(1.0f, -x), x); }
+__device__ __forceinline__ void add_cells(const float *x, const float *d, int n, double &dsum, double &qsum)
 {
-    return __float2bfloat16_rn((float)v);
+    DF ds{0.0f, 0.0f}, qs{0.0f, 0.0f};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        if (e < n) {
+            ds = df_add_acc(ds, df_two_sum(d[e], -x[e]));   // d - x exactly
+            qs = df_add_acc(qs, q_of(x[e]));
+        }
+    dsum += df_to_double(ds);
+    qsum += df_to_double(qs);
 }
 
-// sum of two doubles over the block, result in thread 0
-__device__ __forceinline__ void block_sum2(double &a, double &b)
+// d - alpha q(x), rounded once
+__device__ __forceinline__ double corrected(double d, double x, double alpha, DF)
 {
-    __shared__ double sa[32], sb[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int off = 16; off > 0; off >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, off);
-        b += __shfl_down_sync(0xffffffffu, b, off);
-    }
-    if (lane == 0) {
-        sa[warp] = a;
-        sb[warp] = b;
-    }
+    return d - alpha * (x * (1.0 - x));
+}
+__device__ __forceinline__ float corrected(float d, float x, double, DF alpha)
+{
+    const DF t = df_mul(alpha, q_of(x));
+    const DF s = df_two_sum(d, -t.hi);
+    return __fadd_rn(s.hi, __fsub_rn(s.lo, t.lo));
+}
+
+constexpr int kWarps = 8;   // per block
+
+// sums of a and b over the block's threads, in a of threads 0 and 32
+__device__ __forceinline__ void block_sum2(double &a, double b)
+{
+    __shared__ double s[2][32 * kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    s[0][threadIdx.x] = a;
+    s[1][threadIdx.x] = b;
     __syncthreads();
-    if (warp == 0) {
-        a = lane < nw ? sa[lane] : 0.0;
-        b = lane < nw ? sb[lane] : 0.0;
-        for (int off = 16; off > 0; off >>= 1) {
-            a += __shfl_down_sync(0xffffffffu, a, off);
-            b += __shfl_down_sync(0xffffffffu, b, off);
-        }
+    if (warp < 2) {
+        a = 0.0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) a += s[warp][32 * w + lane];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
     }
 }
+
+// 16 bytes of a row as storage elements
+template <class S> struct Vec {
+    static constexpr int E = 16 / (int)sizeof(S);
+    union {
+        uint4 w;
+        S v[E];
+    };
+    __device__ __forceinline__ Vec() {}
+};
 
 template <class S>
-__global__ void __launch_bounds__(256) conserve_sums_kernel(const GridGeom g, const S *src, const S *dst,
-                                                            double *partials)
+__global__ void __launch_bounds__(32 * kWarps) conserve_sums_kernel(const GridGeom g, const S *src, const S *dst,
+                                                                    double *partials)
 {
+    asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;" ::: "memory");
+    using T = typename Cell<S>::T;
+    constexpr int E = Vec<S>::E;
+    const int lane = threadIdx.x & 31;
     double dsum = 0.0, qsum = 0.0;
-    const long long rows = (long long)g.ny * g.nz;
-    for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-        const long long base = cell_index(g, 0, (int)(row % g.ny), (int)(row / g.ny));
-        for (int i = threadIdx.x; i < g.nx; i += blockDim.x) {
-            const double p = ld64<S>(src, base + i);
-            dsum += ld64<S>(dst, base + i) - p;
-            qsum += p * (1.0 - p);
+    const int rows = g.ny * g.nz;   // a face of the grid is below 2^30 cells
+    for (int row = blockIdx.x * kWarps + (threadIdx.x >> 5); row < rows; row += gridDim.x * kWarps) {
+        const long long base = cell_index(g, 0, row % g.ny, row / g.ny);
+        for (int i = lane * E; i < g.nx; i += 32 * E) {   // rows start on 32 bytes, the pitch covers the last 16
+            Vec<S> p, d;
+            p.w = *reinterpret_cast<const uint4 *>(src + base + i);
+            d.w = *reinterpret_cast<const uint4 *>(dst + base + i);
+            constexpr int G = E < 4 ? E : 4;   // cells of a group
+#pragma unroll
+            for (int e0 = 0; e0 < E; e0 += G) {
+                T x[G], y[G];
+#pragma unroll
+                for (int e = 0; e < G; ++e) {
+                    x[e] = get(p.v[e0 + e]);
+                    y[e] = get(d.v[e0 + e]);
+                }
+                if (i + e0 < g.nx) add_cells(x, y, g.nx - i - e0, dsum, qsum);
+            }
         }
     }
     block_sum2(dsum, qsum);
+    if (threadIdx.x == 0) partials[2 * blockIdx.x] = dsum;
+    if (threadIdx.x == 32) partials[2 * blockIdx.x + 1] = dsum;
+}
+
+// Boundary kinds of the faces as bits (an axis is periodic on both faces or on
+// none) and the signed contact couplings.
+template <class T>
+struct Faces {
+    unsigned periodic, contact;   // bit axis, bit face
+    T a[6];
+};
+
+// The ghost coordinates whose source is c on an axis of n cells, the inverse of
+// map_axis: image 0 is c itself, 1 and 2 the ghosts (kNone: c has none there).
+constexpr int kNone = -2;
+__device__ __forceinline__ int axis_image(int m, int c, int n, bool periodic)
+{
+    if (m == 0) return c;
+    if (m == 1) return (periodic ? c == n - 1 : c == 0) ? -1 : kNone;
+    return (periodic ? c == 0 : c == n - 1) ? n : kNone;
+}
+
+// E cells (i.., j, k) of a row with their stored values v, and the ghosts they
+// are the source of, as the face kernel (boundary.cu) writes them: shifts along
+// x, then y, then z in the compute type (CONTACT: some face has the shift of
+// Eq. 7; without it the images are copies: 4 us less at 60^3).  The y and z images are the warp's, whole rows at a time; most rows
+// have none.
+template <class S, bool CONTACT, int E>
+__device__ __forceinline__ void write_cells(const GridGeom &g, const Faces<typename Cell<S>::T> &fc, S *f,
+                                            const Vec<S> &v, int i, int j, int k)
+{
+    using T = typename Cell<S>::T;
+    auto image = [&](T x, int m, int axis) {
+        const int face = 2 * axis + m - 1;
+        return CONTACT && m > 0 && (fc.contact >> face & 1u) ? contact_shift_rn(x, fc.a[face]) : x;
+    };
+    const bool px = fc.periodic & 1u, py = fc.periodic & 2u, pz = fc.periodic & 4u;
+    const bool edge = j == 0 || j == g.ny - 1 || k == 0 || k == g.nz - 1;
+#pragma unroll 1
+    for (int mz = 0; mz < (edge ? 3 : 1); ++mz) {
+        const int kk = axis_image(mz, k, g.nz, pz);
+        if (kk == kNone) continue;
+#pragma unroll 1
+        for (int my = 0; my < (edge ? 3 : 1); ++my) {
+            const int jj = axis_image(my, j, g.ny, py);
+            if (jj == kNone) continue;
+            auto yz = [&](T x) { return image(image(x, my, 1), mz, 2); };
+            S *row = f + cell_index(g, 0, jj, kk);
+            Vec<S> o;
+            if (CONTACT) {
+#pragma unroll
+                for (int e = 0; e < E; ++e) put(o.v[e], yz(get(v.v[e])));
+            } else {
+                o.w = v.w;
+            }
+            if (i + E <= g.nx) {
+                *reinterpret_cast<uint4 *>(row + i) = o.w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if (i + e < g.nx) row[i + e] = o.v[e];
+            }
+            if (i == 0 || i + E >= g.nx) {   // x ghosts of the row's first and last cell
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int c = i + e;
+                    if (c == 0) {
+                        const int m = px ? 2 : 1;
+                        put(row[px ? g.nx : -1], yz(image(get(v.v[e]), m, 0)));
+                    }
+                    if (c == g.nx - 1) {
+                        const int m = px ? 1 : 2;
+                        put(row[px ? -1 : g.nx], yz(image(get(v.v[e]), m, 0)));
+                    }
+                }
+            }
+        }
+    }
+}
+
+template <class S, bool CONTACT>
+__global__ void __launch_bounds__(32 * kWarps)
+    conserve_apply_kernel(const GridGeom g, const __grid_constant__ Faces<typename Cell<S>::T> fc, const S *src,
+                          S *dst, const double *partials, double *alpha_out)
+{
+    asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;" ::: "memory");
+    constexpr int E = Vec<S>::E;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rows = g.ny * g.nz;
+    __shared__ double s_sum[2];
+    __shared__ DF s_alpha;
+    if (warp < 2) {   // warp 0 the differences, warp 1 the q; all loads under way at once
+        constexpr int kLoads = (kStatsBlocks + 31) / 32;
+        double x[kLoads], v = 0.0;
+#pragma unroll
+        for (int t = 0; t < kLoads; ++t)
+            x[t] = lane + 32 * t < gridDim.x ? partials[2 * (lane + 32 * t) + warp] : 0.0;
+#pragma unroll
+        for (int t = 0; t < kLoads; ++t)
+            if (32 * t < gridDim.x) v += x[t];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+        if (lane == 0) s_sum[warp] = v;
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
-        partials[2 * blockIdx.x] = dsum;
-        partials[2 * blockIdx.x + 1] = qsum;
+        const double al = s_sum[1] != 0.0 ? s_sum[0] / s_sum[1] : 0.0;
+        s_alpha = df_of(al);
+        s_sum[0] = al;
+        if (blockIdx.x == 0) *alpha_out = al;
+    }
+    __syncthreads();
+    const double alpha = s_sum[0];
+    const DF alpha2 = s_alpha;
+    for (int row = blockIdx.x * kWarps + warp; row < rows; row += gridDim.x * kWarps) {
+        const int j = row % g.ny, k = row / g.ny;
+        for (int i = lane * E; i < g.nx; i += 32 * E) {
+            const long long at = cell_index(g, i, j, k);
+            Vec<S> p, d;
+            p.w = *reinterpret_cast<const uint4 *>(src + at);
+            d.w = *reinterpret_cast<const uint4 *>(dst + at);
+#pragma unroll
+            for (int e = 0; e < E; ++e) put(d.v[e], corrected(get(d.v[e]), get(p.v[e]), alpha, alpha2));
+            write_cells<S, CONTACT, E>(g, fc, dst, d, i, j, k);
+        }
     }
 }
 
 template <class S>
-__global__ void __launch_bounds__(256) conserve_apply_kernel(const GridGeom g, const S *src, S *dst,
-                                                             const double *partials, int nblk,
-                                                             double *alpha_out)
+cudaError_t conserve(const GridGeom &g, const double aface[6], const S *src, S *dst, double *partials,
+                     double *alpha_out, cudaStream_t st)
 {
-    __shared__ double s_alpha;
-    if (threadIdx.x == 0) {
-        double d = 0.0, q = 0.0;
-        for (int b = 0; b < nblk; ++b) {   // the same order in every block
-            d += partials[2 * b];
-            q += partials[2 * b + 1];
-        }
-        s_alpha = q != 0.0 ? d / q : 0.0;
-        if (blockIdx.x == 0) *alpha_out = s_alpha;
+    const int rows = g.ny * g.nz, want = (rows + kWarps - 1) / kWarps;
+    const int nblk = want < kStatsBlocks ? want : kStatsBlocks;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(nblk);
+    lc.blockDim = dim3(32 * kWarps);
+    lc.stream = st;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&lc, conserve_sums_kernel<S>, g, src, (const S *)dst, partials);
+    if (e != cudaSuccess) return e;
+    using T = typename Cell<S>::T;
+    Faces<T> fc = {0u, 0u, {}};
+    for (int f = 0; f < 6; ++f) {
+        if (g.bc[f] == SPFM_PERIODIC) fc.periodic |= 1u << (f / 2);
+        if (g.bc[f] == SPFM_CONTACT) fc.contact |= 1u << f;
+        fc.a[f] = (T)aface[f];
     }
-    __syncthreads();
-    const double alpha = s_alpha;
-    const long long rows = (long long)g.ny * g.nz;
-    for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-        const long long base = cell_index(g, 0, (int)(row % g.ny), (int)(row / g.ny));
-        for (int i = threadIdx.x; i < g.nx; i += blockDim.x) {
-            const double p = ld64<S>(src, base + i);
-            dst[base + i] = st_of<S>(ld64<S>(dst, base + i) - alpha * (p * (1.0 - p)));
-        }
-    }
+    if (fc.contact)
+        return cudaLaunchKernelEx(&lc, conserve_apply_kernel<S, true>, g, fc, src, dst,
+                                  (const double *)partials, alpha_out);
+    return cudaLaunchKernelEx(&lc, conserve_apply_kernel<S, false>, g, fc, src, dst,
+                                  (const double *)partials, alpha_out);
 }
 
 }  // namespace
 
-cudaError_t launch_conserve(const GridGeom &g, int dtype, const void *src, void *dst, double *partials,
-                            double *alpha_out, cudaStream_t st)
+cudaError_t launch_conserve(const GridGeom &g, int dtype, const double aface[6], const void *src, void *dst,
+                            double *partials, double *alpha_out, cudaStream_t st)
 {
-    const long long rows = (long long)g.ny * g.nz;
-    const int nblk = (int)(rows < kStatsBlocks ? rows : kStatsBlocks);
-    if (dtype == SPFM_F64) {
-        conserve_sums_kernel<double><<<nblk, 256, 0, st>>>(g, (const double *)src, (const double *)dst, partials);
-        conserve_apply_kernel<double><<<nblk, 256, 0, st>>>(g, (const double *)src, (double *)dst, partials,
-                                                            nblk, alpha_out);
-    } else if (dtype == SPFM_F32) {
-        conserve_sums_kernel<float><<<nblk, 256, 0, st>>>(g, (const float *)src, (const float *)dst, partials);
-        conserve_apply_kernel<float><<<nblk, 256, 0, st>>>(g, (const float *)src, (float *)dst, partials, nblk,
-                                                           alpha_out);
-    } else {
-        conserve_sums_kernel<__nv_bfloat16><<<nblk, 256, 0, st>>>(g, (const __nv_bfloat16 *)src,
-                                                                  (const __nv_bfloat16 *)dst, partials);
-        conserve_apply_kernel<__nv_bfloat16><<<nblk, 256, 0, st>>>(g, (const __nv_bfloat16 *)src,
-                                                                   (__nv_bfloat16 *)dst, partials, nblk,
-                                                                   alpha_out);
-    }
-    return cudaGetLastError();
+    if (dtype == SPFM_F64) return conserve(g, aface, (const double *)src, (double *)dst, partials, alpha_out, st);
+    if (dtype == SPFM_F32) return conserve(g, aface, (const float *)src, (float *)dst, partials, alpha_out, st);
+    return conserve(g, aface, (const __nv_bfloat16 *)src, (__nv_bfloat16 *)dst, partials, alpha_out, st);
 }
 
 }  // namespace spfm

@@ -203,9 +203,10 @@ int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target, bo
 //               itself (no face kernel follows) and lets the next step launch early
 //   kSkipCopy   test of the bounded waits: the first CTA skips one plane's copy
 //               (spfm_debug_skip_copy), its waits give up and set the error word
-//   kEarly      no face kernel follows (no periodic face: the step computes the
-//               ghosts of the non-periodic faces as it reads them): the step lets
-//               the next one launch at its start, like the image-writing kernels
+//   kEarly      the kernel that follows waits for the whole of this one itself (the
+//               next step, where the step computes the ghosts of non-periodic faces as
+//               it reads them; the constant-volume sums): the step lets it launch at
+//               its start, like the image-writing kernels
 constexpr int kWaitFaces = 1, kWaitAll = 2, kImages = 4, kSkipCopy = 8, kEarly = 16;
 
 // TMA tensor maps of a grid's two field buffers, encoded on first use (tma.cu).
@@ -266,10 +267,10 @@ struct InitArgs {
 cudaError_t launch_init(const InitArgs &a, void *field, cudaStream_t st);
 
 // Constant-volume correction after a step at dF = 0 (conserve.cu): dst -=
-// alpha q(src) with alpha = sum(dst - src) / sum q(src); partials holds
-// 2 * kStatsBlocks doubles, alpha_out (device) receives alpha.
-cudaError_t launch_conserve(const GridGeom &g, int dtype, const void *src, void *dst, double *partials,
-                            double *alpha_out, cudaStream_t st);
+// alpha q(src) with alpha = sum(dst - src) / sum q(src), and the ghost layer of
+// dst; partials holds 2 * kStatsBlocks doubles, alpha_out (device) receives alpha.
+cudaError_t launch_conserve(const GridGeom &g, int dtype, const double aface[6], const void *src, void *dst,
+                            double *partials, double *alpha_out, cudaStream_t st);
 
 // Interior of dst = interior of src shifted along x by cells (frame.cu).
 cudaError_t launch_shift_x(const GridGeom &g, int dtype, const void *src, void *dst, int cells, cudaStream_t st);
