@@ -1263,7 +1263,11 @@ cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, 
     if (tmap) map = *tmap;
     else memset(&map, 0, sizeof map);
     const int use = tmap ? 1 : 0;
-    constexpr int R = SPFM_ROWS_PER_THREAD;
+    // Rows per thread: two, and one for BF16, whose threads take eight cells of a
+    // row: with two a CTA had two consumer warps of 168 registers, six an SM
+    // (384^3 TI_<120>, three CTAs per SM: 181 -> 140 us a step with stochastic
+    // rounding, 97 -> 92 without; 64^3 8.6 -> 6.0)
+    constexpr int R = sizeof(S) == 2 ? 1 : SPFM_ROWS_PER_THREAD;
     constexpr int NT1 = TileShape<S, T, TX, TY, 1>::NTHREADS;
     // programmatic dependent launch: the kernel may begin while the previous
     // kernel in the stream runs; cfg.mode says which boxes wait (griddepcontrol)
@@ -1290,7 +1294,7 @@ cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, 
         return cudaLaunchKernelEx(&lc, kern, c, pc, src, dst, err, zchunk, map, use, mode);
     };
     cudaError_t le = cudaSuccess;
-#define SPFM_LAUNCH(ST, KD) le = go(spfm_step_kernel<S, T, ST, KD, TX, TY, R, IMG, SR>, Sh::NTHREADS)
+#define SPFM_LAUNCH(ST, KD) le = go(spfm_step_kernel<S, T, ST, KD, TX, TY, R, IMG, SR>, TileShape<S, T, TX, TY, R>::NTHREADS)
 #define SPFM_BY_KIND(ST)                        \
     do {                                        \
         if (kind == 0) SPFM_LAUNCH(ST, 0);      \
