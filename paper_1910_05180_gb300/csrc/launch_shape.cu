@@ -34,6 +34,16 @@
 // 10.1; 64^3 plane all in the band 16: 40.0, 4: 13.8, 1 (chosen): 7.4; 96^3 16:
 // 46.2, 4 (chosen): 15.5, 2: 16.3; 192^3 16: 72, 4 (chosen): 60.5, 2: 69.8;
 // 256^3 16: 96.0, 8: 90.4 (9 chosen), 4: 94.2; 320^3 16 (chosen): 124.6, 8: 129.
+//
+// The FP64 kernels (CF and TI global) are bound by the FP64 pipe, which the CTAs
+// of an SM share: what counts is the work of the fullest SM, n CTAs on each of
+// at most ceil(CTAs / SMs), a plane of a CTA costing about 9 FP64 instructions a
+// cell as it is read and 18 more as it is written (the halo planes are only
+// read).  One CTA alone keeps the pipe about a third busy, so one or two on an
+// SM take as long as three.  Chunks of 1 to 64 planes, the least work, ties to
+// the longer chunk.  Measured, us a step (planes per CTA): 128 x 32 x 32 7-point
+// 1 (chosen) 16.4, 2: 18.4, 4 (the streaming rule): 18.8; 48^3 1 (chosen) 51.0,
+// 4: 79.2; 96^3 4 (chosen) 110, 2: 125, 12: 264; 256^3 37 (chosen) 1038, 16: 1066.
 #include <map>
 #include <mutex>
 #include <queue>
@@ -107,14 +117,30 @@ static int uneven_zchunk(int tiles, int nz, int slots)
     return zc < 4 ? 4 : (zc > 16 ? 16 : (int)zc);
 }
 
+// planes per CTA of an FP64 launch (see above)
+static int fp64_zchunk(int tiles, int nz, int sms)
+{
+    int best = 1;
+    long long best_work = -1;
+    for (int zc = 1; zc <= (nz < 64 ? nz : 64); ++zc) {
+        const long long ctas = (long long)tiles * ((nz + zc - 1) / zc);
+        const long long n = (ctas + sms - 1) / sms, work = (n < 3 ? 3 : n) * (9 * (zc + 2) + 18 * zc);
+        if (best_work < 0 || work <= best_work) {
+            best_work = work;
+            best = zc;
+        }
+    }
+    return best;
+}
+
 namespace {
 std::mutex g_mu;
-// (kernel, threads, device) -> resident CTAs per SM; (tiles, nz, slots, target or -1: uneven) -> z-chunk
+// (kernel, threads, device) -> resident CTAs per SM; (tiles, nz, slots, target or -family) -> z-chunk
 std::map<std::tuple<const void *, int, int>, int> g_occ;
 std::map<std::tuple<int, int, int, int>, int> g_zc;
 }  // namespace
 
-int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target, bool uneven)
+int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target, int family)
 {
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
@@ -134,11 +160,13 @@ int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target, bo
         g_occ[ok] = per_sm;
     }
     const int slots = per_sm * sms;
-    const auto zk = std::make_tuple(tiles, nz, slots, uneven ? -1 : target);
+    const auto zk = std::make_tuple(tiles, nz, slots, family == kStream ? target : -family);
     auto z = g_zc.find(zk);
     if (z != g_zc.end()) return z->second;
     if (g_zc.size() >= 4096) g_zc.clear();   // many grid shapes (a serving process): start over
-    const int zc = uneven ? uneven_zchunk(tiles, nz, slots) : model_zchunk(tiles, nz, per_sm, slots, target);
+    const int zc = family == kUneven ? uneven_zchunk(tiles, nz, slots)
+                   : family == kFp64 ? fp64_zchunk(tiles, nz, sms)
+                                     : model_zchunk(tiles, nz, per_sm, slots, target);
     g_zc[zk] = zc;
     return zc;
 }

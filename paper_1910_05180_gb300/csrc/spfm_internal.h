@@ -192,9 +192,11 @@ struct LaunchCfg {
 
 // Planes per CTA of a step launch of `tiles` xy tiles over nz planes by kernel
 // `kern` of `threads` threads (launch_shape.cu); target: the CTA count of six
-// rounds at the kernel family's design occupancy; uneven: TI_n, whose CTAs
-// differ in work.  Cached per kernel and shape.
-int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target, bool uneven);
+// rounds at the kernel family's design occupancy; family: the rule (kUneven:
+// TI_n, whose CTAs differ in work; kFp64: bound by an SM's FP64 pipe; else
+// kStream).  Cached per kernel and shape.
+enum { kStream = 0, kUneven = 1, kFp64 = 2 };
+int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target, int family);
 
 // How a step launch sits in the stream (programmatic dependent launch):
 //   kWaitFaces  the previous kernel refreshes src's ghosts: boxes touching a face wait for it

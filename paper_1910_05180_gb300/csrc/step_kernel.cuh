@@ -85,6 +85,10 @@ template <> struct Pk<float> {
         return __fmul2_rn(a, r);
     }
     static __device__ __forceinline__ P rsqrt(P a) { return make_float2(rsqrtf(a.x), rsqrtf(a.y)); }
+    // v (1 - v)
+    static __device__ __forceinline__ P bump(P v, P one) { return mul(v, sub(one, v)); }
+    // a + b - 2 c as the sum of two differences
+    static __device__ __forceinline__ P second(P a, P b, P c) { return add(sub(a, c), sub(b, c)); }
 };
 
 struct D2 { double x, y; };
@@ -99,8 +103,27 @@ template <> struct Pk<double> {
         return {__fma_rn(a.x, b.x, c.x), __fma_rn(a.y, b.y, c.y)};
     }
     static __device__ __forceinline__ P sub(P a, P b) { return {__dsub_rn(a.x, b.x), __dsub_rn(a.y, b.y)}; }
-    static __device__ __forceinline__ P div(P a, P b) { return {a.x / b.x, a.y / b.y}; }
+    // a / b as a * r(b), r(b) the reciprocal by one third-order Newton step from
+    // the hardware's approximation (relative error e < 2^-18, then e^3): 5
+    // instructions of the FP64 pipe, which bounds these kernels, where a division
+    // takes some 14; within 2 ulp for |b| in the normal range, and a zero,
+    // infinite or NaN b gives a non-finite or zero result as the division does
+    static __device__ __forceinline__ double quot(double a, double b)
+    {
+        double r;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
+        const double e = __fma_rn(-b, r, 1.0);
+        return __dmul_rn(a, __fma_rn(__fma_rn(e, e, e), r, r));
+    }
+    static __device__ __forceinline__ P div(P a, P b) { return {quot(a.x, b.x), quot(a.y, b.y)}; }
     static __device__ __forceinline__ P rsqrt(P a) { return {::rsqrt(a.x), ::rsqrt(a.y)}; }
+    // v - v^2, rounded once
+    static __device__ __forceinline__ P bump(P v, P) { return {__fma_rn(-v.x, v.x, v.x), __fma_rn(-v.y, v.y, v.y)}; }
+    // a + b - 2 c, as F' is formed
+    static __device__ __forceinline__ P second(P a, P b, P c)
+    {
+        return {__fma_rn(-2.0, c.x, __dadd_rn(a.x, b.x)), __fma_rn(-2.0, c.y, __dadd_rn(a.y, b.y))};
+    }
 };
 
 template <class T> struct PackT;
@@ -912,11 +935,11 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                     // one by one as that fraction
                     auto pack = [&](int q, auto by_group) -> P {
                         const P ph = z[r].c[q];
-                        const P t = K::add(K::sub(m[r].c[q], ph), K::sub(p[r].c[q], ph));
+                        const P t = K::second(m[r].c[q], p[r].c[q], ph);
                         // SR: the increment alone, phi is added once in sr_update
                         const P acc = laplace_update<SR, STENCIL>(PC, t, ph, z[r].h[q], m[r].g[q], p[r].g[q]);
                         const P sg = K::fma(PC.m2, ph, PC.one);
-                        const P q1 = K::mul(ph, K::sub(PC.one, ph));
+                        const P q1 = K::bump(ph, PC.one);
                         P num, den;
                         if constexpr (by_group.value) {
                             const P u = K::mul(sg, sg);
@@ -1014,11 +1037,11 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
 #pragma unroll
                     for (int q = 0; q < NP; ++q) {
                         const P ph = z[r].c[q];
-                        const P t = K::add(K::sub(m[r].c[q], ph), K::sub(p[r].c[q], ph));
+                        const P t = K::second(m[r].c[q], p[r].c[q], ph);
                         // phi + dt * Laplacian (SR: the increment alone, phi is added in sr_update)
                         const P acc = laplace_update<SR, STENCIL>(PC, t, ph, z[r].h[q], m[r].g[q], p[r].g[q]);
                         const P sg = K::fma(PC.m2, ph, PC.one);               // s = 1 - 2 phi
-                        const P q1 = K::mul(ph, K::sub(PC.one, ph));          // q = phi (1 - phi)
+                        const P q1 = K::bump(ph, PC.one);                     // q = phi (1 - phi)
                         P w;   // -dt (potential / q + 4 M dF / (lambda Gamma))
                         if (KIND == 0) {
                             // driving term -dt pref dF h'(phi) = q (nkmu f): f = 1 for h3,
@@ -1285,7 +1308,7 @@ cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, 
     auto go = [&](auto kern, int threads) {
         int zchunk = cfg.zchunk > 0 ? cfg.zchunk
                                     : pick_zchunk((const void *)kern, threads, gxn * gyn, c.g.nz, target,
-                                                  kind == kKindLocal);
+                                                  kind == kKindLocal ? kUneven : sizeof(T) == 8 ? kFp64 : kStream);
         if (zchunk > c.g.nz) zchunk = c.g.nz;
         if (zchunk < (c.g.nz + 65534) / 65535) zchunk = (c.g.nz + 65534) / 65535;
         if (cfg.zchunk_used) *cfg.zchunk_used = zchunk;
