@@ -296,8 +296,10 @@ spfm_status spfm_batch_step(spfm_batch *b, int n_steps, const spfm_step_args *ar
  *   SPFM_TILES_WIDE    every grid on 64 x 16 tiles
  *   SPFM_TILES_SQUARE  every grid on 32 x 32 tiles
  *   SPFM_TILES_FIT     each grid on the shape that pads its nx x ny extent least,
- *                      ties to 64 x 16 (the default; the two shapes then run as
- *                      two persistent launches per step) */
+ *                      ties to 64 x 16 (the two shapes then run as two
+ *                      persistent launches per step)
+ * A new batch takes the policy and the z-march depth whose CTAs, with the items
+ * dealt to them evenly, have the least work by count of planes. */
 enum { SPFM_TILES_WIDE = 0, SPFM_TILES_SQUARE = 1, SPFM_TILES_FIT = 2 };
 /* Autotuner of the batch's work-list: first the tile policy (FP32 batches: the
  * three above, at the current depth), then the z-march depth of its items

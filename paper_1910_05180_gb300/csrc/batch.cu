@@ -1,17 +1,30 @@
 // batch.cu -- the batch calls of the C ABI.
 //
 // Many grids of one storage type advance together: every step is one launch of
-// the persistent step kernel over a packed tile work-list of all grids (each
-// item: grid, tile column/row, z range of at most kBatchZChunk planes) plus one
-// launch of the ghost-face kernel over all grids.  The per-grid records (step
-// coefficients, buffers, TMA maps) live in the caller's scratch and are read
-// by the kernels at run time, so a captured CUDA graph of kGraphSteps steps is
-// replayed unchanged across calls; parameters can change between calls.  Each
-// grid's arithmetic is exactly the single-grid step's.
+// the persistent step kernel (one per tile shape in use) over a packed tile
+// work-list of all grids (each item: grid, tile column/row, z range of at most
+// `depth` planes), and where a face is periodic one launch of the ghost-face
+// kernel over all grids.  The per-grid records (step coefficients, buffers, TMA
+// maps) live in the caller's scratch and are read by the kernels at run time,
+// so a captured CUDA graph of kGraphSteps steps is replayed unchanged across
+// calls; parameters can change between calls.  Each grid's arithmetic is
+// exactly the single-grid step's.
+//
+// Balance.  The items are dealt to the CTAs on the host, longest first, each
+// to the CTA with the least work so far (an item costs its planes + 3: two halo
+// planes and its start).  The default tile policy and depth are the ones whose
+// fullest CTA has the least work, over the launches of a step.  us a step,
+// FP32 13 groups: 64 grids of 32 to 96 cells 92 (fixed depth 32, each grid on
+// its best-fitting shape, items dealt in turn) -> 80; 32 grids of 32 to 192
+// cells, stochastic rounding, 346 -> 290.  Both shapes side by side, as two
+// branches of the graph with the slots split by their work, ran 92 and 383:
+// two kernels on one SM evict each other's instructions.
 #include <math.h>
 #include <string.h>
 
 #include <algorithm>
+#include <queue>
+#include <utility>
 #include <vector>
 
 #include "host_internal.h"
@@ -21,17 +34,17 @@ using namespace spfm_host;
 
 namespace {
 
-constexpr int kBatchZChunk = 32;   // z-march depth of the items until tuned
 constexpr int kGraphSteps = 16;    // steps per captured graph (even: parity repeats)
 // depths the autotuner tries; the scratch holds the work-list of the shallowest
 constexpr int kDepths[] = {8, 12, 16, 24, 32, 48, 64};
 constexpr int kNDepths = (int)(sizeof(kDepths) / sizeof(kDepths[0]));
 constexpr int kMinDepth = 8;
+constexpr int kMaxCtas = 1024;   // of one launch
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Layout {
-    size_t grids, items, ghosts, stats_jobs, partials, finals, err, steps, total;
+    size_t grids, items, starts, ghosts, stats_jobs, partials, finals, err, steps, total;
 };
 
 size_t grid_record_bytes(int dtype)
@@ -69,6 +82,8 @@ Layout layout_for(int dtype, int n, int nitems)
     off = align_up(off + grid_record_bytes(dtype) * n, 256);
     L.items = off;
     off = align_up(off + sizeof(BatchItem) * nitems, 256);
+    L.starts = off;   // first item of every CTA, both shapes
+    off = align_up(off + sizeof(int) * 2 * (kMaxCtas + 1), 256);
     L.ghosts = off;
     off = align_up(off + sizeof(GhostJob) * n, 256);
     L.stats_jobs = off;
@@ -108,12 +123,14 @@ int check_grids(spfm_grid *const *grids, int n, int *dtype, int *nitems)
 
 struct spfm_batch {
     std::vector<spfm_grid *> grids;
-    int n = 0, dtype = 0, nitems = 0, depth = kBatchZChunk, policy = SPFM_TILES_FIT;
-    int nitems0 = 0;   // items of shape 0; the shape-1 items follow them in the list
+    int n = 0, dtype = 0, depth = 0, policy = SPFM_TILES_FIT;
+    int ctas[2] = {0, 0};     // CTAs of each shape's launch
+    int nitems0 = 0;          // items of shape 0; the shape-1 items follow them in the list
     char *scratch = nullptr;
     cudaStream_t stream = nullptr;
     Layout L;
     std::vector<BatchItem> h_items;
+    std::vector<int> h_starts;
     std::vector<char> h_grids;
     std::vector<GhostJob> h_ghosts;
     std::vector<StatsJob> h_stats;
@@ -138,66 +155,141 @@ static int bfail(spfm_batch *b, int code, const char *msg)
     return fail(nullptr, code, "%s", msg);
 }
 
-// the work-list of z-march depth `depth` under the batch's tile policy,
-// uploaded on the batch's stream (the captured graph holds the item count, so
-// it is dropped)
-static cudaError_t set_depth(spfm_batch *b, int depth)
+// The items of a tile policy and depth, dealt to CTAs.
+struct Deal {
+    std::vector<BatchItem> items;   // in CTA order, shape 0 first
+    std::vector<int> starts;        // kMaxCtas + 1 entries a shape
+    int ctas[2] = {0, 0}, nitems0 = 0;
+    long long span = 0;             // work of the fullest CTA, summed over the launches of a step
+};
+
+static void deal_items(const spfm_batch *b, int policy, int depth, int slots, Deal &d)
 {
-    int k = 0;
+    constexpr int kStart = 3;   // halo planes and start of an item, in planes
+    std::vector<BatchItem> list[2];
     for (int i = 0; i < b->n; ++i) {
         const GridGeom &g = b->grids[i]->geom;
-        k += items_of(b->dtype, g, i, depth, nullptr, shape_for(b->dtype, g, b->policy));
+        const int shape = shape_for(b->dtype, g, policy);
+        std::vector<BatchItem> &l = list[shape];
+        const size_t at = l.size();
+        l.resize(at + items_of(b->dtype, g, i, depth, nullptr, shape));
+        items_of(b->dtype, g, i, depth, l.data() + at, shape);
     }
-    b->h_items.resize(k);
-    k = 0;
-    for (int shape = 0; shape < 2; ++shape) {   // shape 0 items first, one launch per shape
-        for (int i = 0; i < b->n; ++i) {
-            const GridGeom &g = b->grids[i]->geom;
-            if (shape_for(b->dtype, g, b->policy) == shape)
-                k += items_of(b->dtype, g, i, depth, b->h_items.data() + k, shape);
+    slots = std::min(slots, kMaxCtas);
+    for (int s = 0; s < 2; ++s) d.ctas[s] = (int)std::min<size_t>(list[s].size(), slots);
+    d.items.clear();
+    d.starts.assign(2 * (kMaxCtas + 1), 0);
+    d.span = 0;
+    for (int s = 0; s < 2; ++s) {
+        std::vector<BatchItem> &l = list[s];
+        const int ctas = d.ctas[s];
+        // longest first (stable: neighbouring tiles stay together), to the least loaded
+        std::stable_sort(l.begin(), l.end(), [](const BatchItem &x, const BatchItem &y) {
+            return x.zc1 - x.zc0 > y.zc1 - y.zc0;
+        });
+        std::vector<int> owner(l.size()), count(ctas + 1, 0);
+        std::priority_queue<std::pair<long long, int>, std::vector<std::pair<long long, int>>,
+                            std::greater<std::pair<long long, int>>> least;
+        for (int c = 0; c < ctas; ++c) least.push({0, c});
+        long long span = 0;
+        for (size_t k = 0; k < l.size(); ++k) {
+            std::pair<long long, int> t = least.top();
+            least.pop();
+            owner[k] = t.second;
+            ++count[t.second + 1];
+            t.first += l[k].zc1 - l[k].zc0 + kStart;
+            span = std::max(span, t.first);
+            least.push(t);
         }
-        if (shape == 0) b->nitems0 = k;
+        int *start = d.starts.data() + s * (kMaxCtas + 1);
+        for (int c = 0; c < ctas; ++c) start[c + 1] = start[c] + count[c + 1];
+        const size_t at = d.items.size();
+        d.items.resize(at + l.size());
+        std::vector<int> next(start, start + ctas);
+        for (size_t k = 0; k < l.size(); ++k) d.items[at + next[owner[k]]++] = l[k];
+        if (s == 0) d.nitems0 = (int)l.size();
+        d.span += span;
     }
-    b->nitems = k;
+}
+
+// The work-list of z-march depth `depth` under the batch's tile policy (0: the
+// policy and depth with the least span), uploaded on the batch's stream (the
+// captured graph holds the launch sizes, so it is dropped).
+static cudaError_t set_depth(spfm_batch *b, int depth)
+{
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int slots = sms * kBatchCtasPerSm;
+    Deal d;
+    if (depth == 0) {
+        long long best = -1;
+        Deal t;
+        for (int p = 0; p < (b->dtype == SPFM_F32 ? 3 : 1); ++p)
+            for (int c = kNDepths - 1; c >= 0; --c) {
+                const int policy = b->dtype == SPFM_F32 ? p : b->policy;
+                deal_items(b, policy, kDepths[c], slots, t);
+                const bool many = (long long)t.items.size() > 12LL * slots;
+                if (best < 0 || t.span < best || (t.span == best && b->policy == policy)) {
+                    best = t.span;
+                    depth = kDepths[c];
+                    b->policy = policy;
+                    std::swap(d, t);
+                }
+                if (many) break;   // shorter items would only add halo planes
+            }
+    } else {
+        deal_items(b, b->policy, depth, slots, d);
+    }
     b->depth = depth;
+    b->nitems0 = d.nitems0;
+    for (int s = 0; s < 2; ++s) b->ctas[s] = d.ctas[s];
+    b->h_items.swap(d.items);
+    b->h_starts.swap(d.starts);
     if (b->exec) {
         cudaGraphExecDestroy(b->exec);
         b->exec = nullptr;
     }
-    return cudaMemcpyAsync(b->scratch + b->L.items, b->h_items.data(), sizeof(BatchItem) * k,
-                           cudaMemcpyHostToDevice, b->stream);
+    cudaError_t e = cudaMemcpyAsync(b->scratch + b->L.items, b->h_items.data(), sizeof(BatchItem) * b->h_items.size(),
+                                    cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->scratch + b->L.starts, b->h_starts.data(), sizeof(int) * b->h_starts.size(),
+                            cudaMemcpyHostToDevice, b->stream);
+    return e;
 }
 
-// one step of every grid: persistent step kernel (one per tile shape in the
-// list), then the ghost faces of the buffers it wrote; sub: the step's index
-// since the device step counters were last advanced
-static cudaError_t launch_one(spfm_batch *b, int parity, int stencil, int kind, int sub)
+// one step of the grids of one tile shape; sub: the step's index since
+// the device step counters were last advanced
+static cudaError_t launch_shape(spfm_batch *b, int shape, int parity, int stencil, int kind, int sub)
 {
+    if (b->ctas[shape] == 0) return cudaSuccess;
     const void *grids = b->scratch + b->L.grids;
-    const BatchItem *items = (const BatchItem *)(b->scratch + b->L.items);
     int *err = (int *)(b->scratch + b->L.err);
     const long long *steps = (const long long *)(b->scratch + b->L.steps);
-    cudaError_t e;
+    const BatchList list = {(const BatchItem *)(b->scratch + b->L.items) + (shape ? b->nitems0 : 0),
+                            (const int *)(b->scratch + b->L.starts) + shape * (kMaxCtas + 1), b->ctas[shape]};
     const int fwd = b->inline_faces ? 1 : 0;
-    if (b->dtype == SPFM_F64) {
-        e = launch_batch_f64(grids, items, b->nitems, parity, err, stencil, kind, b->stream, fwd);
-    } else if (b->dtype == SPFM_F32) {
-        // the two tile shapes run as two persistent launches over their parts of
-        // the list (their grids differ, so the second needs nothing of the first)
-        e = cudaSuccess;
-        if (b->nitems0 > 0)
-            e = launch_batch_f32(grids, items, b->nitems0, parity, err, stencil, kind, b->stream, 0, b->sr, steps,
-                                 sub, fwd);
-        if (e == cudaSuccess && b->nitems > b->nitems0)
-            e = launch_batch_f32(grids, items + b->nitems0, b->nitems - b->nitems0, parity, err, stencil, kind,
-                                 b->stream, 1, b->sr, steps, sub, fwd);
-    } else {
-        e = launch_batch_bf16(grids, items, b->nitems, parity, err, stencil, kind, b->stream, b->sr, steps, sub,
-                              fwd);
+    const cudaStream_t st = b->stream;
+    if (b->dtype == SPFM_F64) return launch_batch_f64(grids, list, parity, err, stencil, kind, st, fwd);
+    if (b->dtype == SPFM_F32)
+        return launch_batch_f32(grids, list, parity, err, stencil, kind, st, shape, b->sr, steps, sub, fwd);
+    return launch_batch_bf16(grids, list, parity, err, stencil, kind, st, b->sr, steps, sub, fwd);
+}
+
+// n steps of every grid from parity first & 1, each followed by the ghost faces
+// of the buffers it wrote where a face is periodic
+static cudaError_t launch_steps(spfm_batch *b, int first, int n, int stencil, int kind)
+{
+    cudaError_t e = cudaSuccess;
+    for (int s = 0; s < n && e == cudaSuccess; ++s) {
+        const int parity = (first + s) & 1;
+        for (int shape = 0; shape < 2 && e == cudaSuccess; ++shape)
+            e = launch_shape(b, shape, parity, stencil, kind, s);
+        if (e == cudaSuccess && !b->inline_faces)
+            e = launch_fill_ghosts_batch((const GhostJob *)(b->scratch + b->L.ghosts), b->n, b->dtype, parity ^ 1,
+                                         b->stream);
     }
-    if (e != cudaSuccess || b->inline_faces) return e;
-    return launch_fill_ghosts_batch((const GhostJob *)(b->scratch + b->L.ghosts), b->n, b->dtype,
-                                    parity ^ 1, b->stream);
+    return e;
 }
 
 static cudaError_t capture_graph(spfm_batch *b, int stencil, int kind)
@@ -210,8 +302,7 @@ static cudaError_t capture_graph(spfm_batch *b, int stencil, int kind)
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    cudaError_t le = cudaSuccess;
-    for (int s = 0; s < kGraphSteps && le == cudaSuccess; ++s) le = launch_one(b, s & 1, stencil, kind, s);
+    cudaError_t le = launch_steps(b, 0, kGraphSteps, stencil, kind);
     if (le == cudaSuccess && b->sr)
         le = launch_advance_steps((long long *)(b->scratch + b->L.steps), b->n, kGraphSteps, b->stream);
     e = cudaStreamEndCapture(b->stream, &graph);
@@ -270,7 +361,6 @@ spfm_status spfm_batch_create(spfm_grid *const *grids, int n, void *scratch, siz
     b->grids.assign(grids, grids + n);
     b->n = n;
     b->dtype = dtype;
-    b->nitems = nitems;
     b->scratch = (char *)scratch;
     b->stream = (cudaStream_t)stream;
     b->L = L;
@@ -281,7 +371,7 @@ spfm_status spfm_batch_create(spfm_grid *const *grids, int n, void *scratch, siz
     b->h_stats.resize(n);
     b->h_finals.resize((size_t)kNStat * n + 1);
     b->h_steps.resize(n);
-    cudaError_t e = set_depth(b, kBatchZChunk);
+    cudaError_t e = set_depth(b, 0);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->scratch + L.err, 0, 16, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) {
@@ -365,8 +455,8 @@ spfm_status spfm_batch_step(spfm_batch *b, int n_steps, const spfm_step_args *ar
         }
     }
     const int s0 = s;   // the graphs advanced the device step counters up to here
-    for (; s < n_steps; ++s) {
-        e = launch_one(b, s & 1, stencil, kind, s - s0);
+    if (s < n_steps) {
+        e = launch_steps(b, s, n_steps - s, stencil, kind);
         if (e != cudaSuccess) return bfail(b, SPFM_ECUDA, cudaGetErrorString(e));
     }
     if (b->sr && n_steps > s0) {
@@ -435,7 +525,7 @@ spfm_status spfm_batch_autotune(spfm_batch *b, const spfm_step_args *args, int s
         }
         b->policy = best_policy;
     }
-    int best = kBatchZChunk;
+    int best = b->depth;
     double best_ms = 0.0;
     for (int c = 0; c < kNDepths && st == SPFM_OK; ++c) {
         e = set_depth(b, kDepths[c]);

@@ -311,6 +311,15 @@ struct BatchItem {
     int shape;   // tile shape of the item (0: the single-grid shape; 1: the square FP32 shape)
 };
 
+// The items of one tile shape as a launch takes them: CTA b of ctas computes
+// work[start[b]] .. work[start[b + 1] - 1] (device memory).
+struct BatchList {
+    const BatchItem *work;
+    const int *start;
+    int ctas;
+};
+constexpr int kBatchCtasPerSm = 3;   // resident CTAs of the batch kernels (four: 96 registers, spills, 6-11 % slower)
+
 // Per-dtype pieces of the persistent batch kernel (step_f32.cu / ...):
 // bytes of one device-side grid record, the work-list items of one grid, the
 // record of one grid, and the launch of one step over the whole work-list
@@ -330,18 +339,18 @@ void batch_fill_grid_bf16(void *slot, const StepCoef<float> &c, void *const fiel
 // (the launch's position in the call)
 // fwd: no grid of the batch has a periodic face; the kernel stages the ghosts
 // of the faces and no ghost kernel has to run
-cudaError_t launch_batch_f32(const void *grids, const BatchItem *work, int nwork, int parity, int *err,
+cudaError_t launch_batch_f32(const void *grids, BatchList list, int parity, int *err,
                              int stencil, int kind, cudaStream_t st, int shape, int sr, const long long *steps,
                              int sub, int fwd);
-cudaError_t launch_batch_f64(const void *grids, const BatchItem *work, int nwork, int parity, int *err,
+cudaError_t launch_batch_f64(const void *grids, BatchList list, int parity, int *err,
                              int stencil, int kind, cudaStream_t st, int fwd);
-cudaError_t launch_batch_bf16(const void *grids, const BatchItem *work, int nwork, int parity, int *err,
+cudaError_t launch_batch_bf16(const void *grids, BatchList list, int parity, int *err,
                               int stencil, int kind, cudaStream_t st, int sr, const long long *steps, int sub,
                               int fwd);
-cudaError_t launch_batch_f32_sr(const void *grids, const BatchItem *work, int nwork, int parity, int *err,
+cudaError_t launch_batch_f32_sr(const void *grids, BatchList list, int parity, int *err,
                                 int stencil, int kind, cudaStream_t st, int shape, const long long *steps, int sub,
                                 int fwd);
-cudaError_t launch_batch_bf16_sr(const void *grids, const BatchItem *work, int nwork, int parity, int *err,
+cudaError_t launch_batch_bf16_sr(const void *grids, BatchList list, int parity, int *err,
                                  int stencil, int kind, cudaStream_t st, const long long *steps, int sub, int fwd);
 // steps[i] += k for the n grids of a batch (after the k steps of a call or graph)
 cudaError_t launch_advance_steps(long long *steps, int n, int k, cudaStream_t st);

@@ -13,10 +13,10 @@ cudaError_t launch_step_bf16_sr(const StepCoef<float> &c, const __nv_bfloat16 *s
     return launch_step_t<__nv_bfloat16, float, kBfTX, kBfTY, false, true>(c, src, dst, err, cfg, map, st);
 }
 
-cudaError_t launch_batch_bf16_sr(const void *grids, const BatchItem *work, int nwork, int parity, int *err,
+cudaError_t launch_batch_bf16_sr(const void *grids, BatchList list, int parity, int *err,
                                  int stencil, int kind, cudaStream_t st, const long long *steps, int sub, int fwd)
 {
-    return launch_batch_t<__nv_bfloat16, float, kBfTX, kBfTY, false, true>(grids, work, nwork, parity, err,
+    return launch_batch_t<__nv_bfloat16, float, kBfTX, kBfTY, false, true>(grids, list, parity, err,
                                                                            stencil, kind, st, steps, sub, fwd);
 }
 }  // namespace spfm

@@ -13,14 +13,14 @@ cudaError_t launch_step_f32_sr(const StepCoef<float> &c, const float *src, float
     return launch_step_t<float, float, SPFM_F32_TX, SPFM_F32_TY, false, true>(c, src, dst, err, cfg, map, st);
 }
 
-cudaError_t launch_batch_f32_sr(const void *grids, const BatchItem *work, int nwork, int parity, int *err,
+cudaError_t launch_batch_f32_sr(const void *grids, BatchList list, int parity, int *err,
                                 int stencil, int kind, cudaStream_t st, int shape, const long long *steps, int sub,
                                 int fwd)
 {
     if (shape == 1)
-        return launch_batch_t<float, float, kSqTX, kSqTY, true, true>(grids, work, nwork, parity, err, stencil,
+        return launch_batch_t<float, float, kSqTX, kSqTY, true, true>(grids, list, parity, err, stencil,
                                                                        kind, st, steps, sub, fwd);
-    return launch_batch_t<float, float, SPFM_F32_TX, SPFM_F32_TY, false, true>(grids, work, nwork, parity, err,
+    return launch_batch_t<float, float, SPFM_F32_TX, SPFM_F32_TY, false, true>(grids, list, parity, err,
                                                                                stencil, kind, st, steps, sub, fwd);
 }
 }  // namespace spfm

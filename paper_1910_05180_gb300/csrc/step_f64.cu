@@ -38,10 +38,10 @@ void batch_fill_grid_f64(void *slot, const StepCoef<double> &c, void *const fiel
     b->has_map_sq = 0;
 }
 
-cudaError_t launch_batch_f64(const void *grids, const BatchItem *work, int nwork, int parity,
+cudaError_t launch_batch_f64(const void *grids, BatchList list, int parity,
                               int *err, int stencil, int kind, cudaStream_t st, int fwd)
 {
-    return launch_batch_t<double, double, 16, 16>(grids, work, nwork, parity, err, stencil, kind, st, nullptr, 0,
+    return launch_batch_t<double, double, 16, 16>(grids, list, parity, err, stencil, kind, st, nullptr, 0,
                                                   fwd);
 }
 }  // namespace spfm

@@ -1121,7 +1121,6 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
 // spill there, and the persistent batch kernel keeps three.
 template <class S> struct MinBlocks { static constexpr int value = SPFM_MIN_CTAS; };
 template <> struct MinBlocks<float> { static constexpr int value = 4; };
-template <class S> struct BatchMinBlocks { static constexpr int value = SPFM_MIN_CTAS; };
 
 // (the stochastic-rounding kernels and the potentials with the guard on q keep
 // three CTAs per SM: at four their registers spill; 150 x 133 x 117 with a
@@ -1180,15 +1179,16 @@ struct BatchGrid {
 };
 
 // Persistent kernel over a packed work-list of items of one tile shape (TX,
-// TY): CTA b takes items b, b + gridDim.x, ...  Step `parity` reads buffer
-// cur ^ parity.  SQ: the items use the square tile's TMA maps (map_sq).
+// TY): CTA b takes items start[b] .. start[b + 1] - 1 (batch.cu balances
+// them).  Step `parity` reads buffer cur ^ parity.  Every thread waits for the
+// launch before (programmatic dependent launch: the next step's CTAs take the
+// slots that this one's leave).  SQ: the items use the square tile's TMA maps (map_sq).
 // SR: stochastic rounding, the step key of grid i from sr_step_key(its seed,
 // steps[i] + sub).  fwd: no grid of the batch has a periodic face (the
 // producer warp stages the ghosts of the faces; no ghost kernel runs).
 template <class S, class T, int STENCIL, int KIND, int TX, int TY, bool SQ, bool SR = false>
-__global__ void __launch_bounds__(TileShape<S, T, TX, TY>::NTHREADS, BatchMinBlocks<S>::value)
-    spfm_batch_kernel(const BatchGrid<T> *__restrict__ grids, const BatchItem *__restrict__ work,
-                      int nwork, int parity, int *__restrict__ err, const long long *__restrict__ steps,
+__global__ void __launch_bounds__(TileShape<S, T, TX, TY>::NTHREADS, kBatchCtasPerSm)
+    spfm_batch_kernel(const BatchGrid<T> *__restrict__ grids, const BatchList list, int parity, int *__restrict__ err, const long long *__restrict__ steps,
                       int sub, int fwd)
 {
     using Sh = TileShape<S, T, TX, TY>;
@@ -1203,15 +1203,17 @@ __global__ void __launch_bounds__(TileShape<S, T, TX, TY>::NTHREADS, BatchMinBlo
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;" ::: "memory");
     int base = 0;
-    for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
-        const BatchItem it = work[w];
+    const int end = list.start[blockIdx.x + 1];
+    for (int w = list.start[blockIdx.x]; w < end; ++w) {
+        const BatchItem it = list.work[w];
         const BatchGrid<T> &bg = grids[it.grid];
         const int cur = bg.cur ^ parity;
         const CUtensorMap *map = SQ ? (bg.has_map_sq ? &bg.map_sq[cur] : nullptr) : (bg.has_map ? &bg.map[cur] : nullptr);
         if (map && threadIdx.x == Sh::NCONS)
             asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(map) : "memory");
-        const bool last = w + (int)gridDim.x >= nwork;
+        const bool last = w + 1 == end;
         const uint32_t key = SR ? sr_step_key(bg.C.sr_seed, steps[it.grid] + sub) : 0u;
         if (!step_tile<S, T, STENCIL, KIND, TX, TY, SPFM_ROWS_PER_THREAD, false, SR>(
                 bg.C, bg.PC, (const S *)bg.field[cur], (S *)bg.field[cur ^ 1], err, map, it.bx, it.by, it.zc0,
@@ -1239,21 +1241,26 @@ inline int batch_items_t(const GridGeom &g, int grid_index, int zchunk, BatchIte
 }
 
 template <class S, class T, int TX, int TY, bool SQ = false, bool SR = false>
-cudaError_t launch_batch_t(const void *grids, const BatchItem *work, int nwork, int parity, int *err,
+cudaError_t launch_batch_t(const void *grids, BatchList list, int parity, int *err,
                            int stencil, int kind, cudaStream_t st, const long long *steps = nullptr,
                            int sub = 0, int fwd = 0)
 {
     using Sh = TileShape<S, T, TX, TY>;
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int ctas = sms * BatchMinBlocks<S>::value;
-    if (ctas > nwork) ctas = nwork;
-    if (ctas < 1) return cudaSuccess;
+    if (list.ctas < 1) return cudaSuccess;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(list.ctas);
+    lc.blockDim = dim3(Sh::NTHREADS);
+    lc.stream = st;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    cudaError_t le = cudaSuccess;
     const BatchGrid<T> *bg = (const BatchGrid<T> *)grids;
-#define SPFM_BLAUNCH(ST, KD)                                                                               \
-    spfm_batch_kernel<S, T, ST, KD, TX, TY, SQ, SR><<<ctas, Sh::NTHREADS, 0, st>>>(bg, work, nwork, parity, err, \
-                                                                                 steps, sub, fwd)
+#define SPFM_BLAUNCH(ST, KD)                                                                                \
+    le = cudaLaunchKernelEx(&lc, spfm_batch_kernel<S, T, ST, KD, TX, TY, SQ, SR>, bg, list, parity, err, steps, sub, \
+                            fwd)
 #define SPFM_BBY_KIND(ST)                      \
     do {                                       \
         if (kind == 0) SPFM_BLAUNCH(ST, 0);    \
@@ -1266,6 +1273,7 @@ cudaError_t launch_batch_t(const void *grids, const BatchItem *work, int nwork, 
     else SPFM_BBY_KIND(26);
 #undef SPFM_BBY_KIND
 #undef SPFM_BLAUNCH
+    if (le != cudaSuccess) return le;
     return cudaGetLastError();
 }
 
