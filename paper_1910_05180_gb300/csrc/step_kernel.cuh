@@ -71,6 +71,7 @@ template <class T> struct Pk;
 template <> struct Pk<float> {
     using P = float2;
     static __device__ __forceinline__ P mk(float a, float b) { return make_float2(a, b); }
+    static __device__ __forceinline__ float add1(float a, float b) { return __fadd_rn(a, b); }
     static __device__ __forceinline__ P add(P a, P b) { return __fadd2_rn(a, b); }
     static __device__ __forceinline__ P mul(P a, P b) { return __fmul2_rn(a, b); }
     static __device__ __forceinline__ P fma(P a, P b, P c) { return __ffma2_rn(a, b, c); }
@@ -96,6 +97,7 @@ struct D2 { double x, y; };
 template <> struct Pk<double> {
     using P = D2;
     static __device__ __forceinline__ P mk(double a, double b) { return {a, b}; }
+    static __device__ __forceinline__ double add1(double a, double b) { return __dadd_rn(a, b); }
     static __device__ __forceinline__ P add(P a, P b) { return {__dadd_rn(a.x, b.x), __dadd_rn(a.y, b.y)}; }
     static __device__ __forceinline__ P mul(P a, P b) { return {__dmul_rn(a.x, b.x), __dmul_rn(a.y, b.y)}; }
     static __device__ __forceinline__ P fma(P a, P b, P c)
@@ -573,23 +575,14 @@ __device__ __forceinline__ typename Pk<T>::P ti_local_w(const StepCoef<T> &C, ty
     return K::mk(g2.x >= lim ? w.x : wcf.x, g2.y >= lim ? w.y : wcf.y);
 }
 
-// The packs of one staged row around a thread's cells (adjacent pairs):
-// c[p] = (x+2p, x+2p+1), w[p] = c shifted by -1, e[p] = shifted by +1.
+// One staged row around a thread's cells: v[0] the cell to their left, v[1..VX]
+// the cells, v[VX + 1] the one to their right.
 template <class S, class T, int VX>
-__device__ __forceinline__ void get_row(const S *r, typename Pk<T>::P *c, typename Pk<T>::P *w,
-                                        typename Pk<T>::P *e)
+__device__ __forceinline__ void get_row(const S *r, T *v)
 {
-    using K = Pk<T>;
-    T v[VX + 2];
     Io<S, T>::lds(r, v + 1);
     v[0] = Io<S, T>::cvt_in(r[-1]);
     v[VX + 1] = Io<S, T>::cvt_in(r[VX]);
-#pragma unroll
-    for (int p = 0; p < VX / 2; ++p) {
-        c[p] = K::mk(v[2 * p + 1], v[2 * p + 2]);
-        w[p] = K::mk(v[2 * p], v[2 * p + 1]);
-        e[p] = K::mk(v[2 * p + 2], v[2 * p + 3]);
-    }
 }
 
 // Periodic images across the z faces of the 16 bytes of new cells at
@@ -839,7 +832,7 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
     const int gx = x0 + tx * VX;
     const int gy = y0 + ty;
     const S *rbase = stages + (ty + 1) * SW + VX + tx * VX;   // first own row in a stage
-    S *obase = dst + cell_index(g, gx, gy, 0);                // plane 0, first own row
+    S *out = dst + cell_index(g, gx, gy, zc0);                // first own row of the output plane
     // Periodic images (IMG: all faces periodic, nx a multiple of 2 VX, nx >= 4 VX,
     // ny >= 2): a cell in the first two 16-byte chunks of a row also goes to the
     // sector right of the row (x + nx), one in the last two chunks to the sector
@@ -854,6 +847,8 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
     bool img = false;
     if constexpr (IMG) img = gx < 2 * VX || gx >= g.nx - 2 * VX || gy == 0 || gy + RPT >= g.ny;
 
+    const int rows = gx < g.nx ? min(RPT, g.ny - gy) : 0;   // own rows inside the grid
+    const bool whole = gx + VX <= g.nx;
     bool ok = true;
     auto body = [&](int i, PlaneQ<T, NP> (&m)[RPT], PlaneQ<T, NP> (&z)[RPT],
                     PlaneQ<T, NP> (&p)[RPT]) -> bool {
@@ -867,9 +862,17 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
         {
             // rows ty-1 .. ty+RPT of the stage (north halo, own rows, south halo)
             const S *r0 = rbase + s * STAGE - SW;
-            P rc[RPT + 2][NP], rw[RPT + 2][NP], re[RPT + 2][NP];
+            T v[RPT + 2][VX + 2];
 #pragma unroll
-            for (int r = 0; r < RPT + 2; ++r) get_row<S, T, VX>(r0 + r * SW, rc[r], rw[r], re[r]);
+            for (int r = 0; r < RPT + 2; ++r) get_row<S, T, VX>(r0 + r * SW, v[r]);
+            // a pack of row r, and the sums W + E of its cells: the left and right
+            // neighbours straddle register pairs, so they are added one by one
+            // instead of being moved into packs (512^3 TI_<120> 194.9 -> 188.7 us,
+            // 384^3 BF16 with stochastic rounding 139.7 -> 127.7)
+            auto cell = [&](int r, int q) { return K::mk(v[r][2 * q + 1], v[r][2 * q + 2]); };
+            auto side = [&](int r, int q) {
+                return K::mk(K::add1(v[r][2 * q], v[r][2 * q + 2]), K::add1(v[r][2 * q + 1], v[r][2 * q + 3]));
+            };
             // TI_n reads the plane's neighbours again when it is the centre plane, and
             // releases it then
             if constexpr (KIND != kKindLocal) {
@@ -879,17 +882,17 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                 int hi[RPT + 2], lo[RPT + 2];
 #pragma unroll
                 for (int r = 0; r < RPT + 2; ++r) {
-                    hi[r] = lo[r] = (int)top_bits(rc[r][0].x);
+                    hi[r] = lo[r] = (int)top_bits(v[r][1]);
 #pragma unroll
-                    for (int e = 1; e < VX; ++e) {
-                        const int b = (int)top_bits(e & 1 ? rc[r][e / 2].y : rc[r][e / 2].x);
+                    for (int e = 2; e <= VX; ++e) {
+                        const int b = (int)top_bits(v[r][e]);
                         hi[r] = max(hi[r], b);
                         lo[r] = min(lo[r], b);
                     }
                 }
 #pragma unroll
                 for (int r = 0; r < RPT; ++r) {
-                    const int w = (int)top_bits(rw[r + 1][0].x), e = (int)top_bits(re[r + 1][NP - 1].y);
+                    const int w = (int)top_bits(v[r + 1][0]), e = (int)top_bits(v[r + 1][VX + 1]);
                     p[r].own = clamp_level(hi[r + 1], lo[r + 1], C.eps);
                     p[r].level = clamp_level(max(max(max(hi[r], hi[r + 1]), hi[r + 2]), max(w, e)),
                                              min(min(min(lo[r], lo[r + 1]), lo[r + 2]), min(w, e)), C.eps);
@@ -899,18 +902,16 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
             for (int r = 0; r < RPT; ++r) {
 #pragma unroll
                 for (int q = 0; q < NP; ++q) {
-                    const P c = rc[r + 1][q];
+                    const P c = cell(r + 1, q);
                     p[r].c[q] = c;
                     // F' = (W + E + N + S) - 4C, E' = (NW + NE + SW + SE) - 4C
-                    const P f = K::fma(PC.m4, c, K::add(K::add(rw[r + 1][q], re[r + 1][q]),
-                                                        K::add(rc[r][q], rc[r + 2][q])));
+                    const P f = K::fma(PC.m4, c, K::add(side(r + 1, q), K::add(cell(r, q), cell(r + 2, q))));
                     // 6 neighbours: h = F' (c1 applied in the update's FMA); 18: g = F'
                     // (c2 applied to the sum of the two planes' g in one FMA)
                     if (STENCIL == 6) {
                         p[r].h[q] = f;
                     } else {
-                        const P e = K::fma(PC.m4, c, K::add(K::add(rw[r][q], re[r][q]),
-                                                            K::add(rw[r + 2][q], re[r + 2][q])));
+                        const P e = K::fma(PC.m4, c, K::add(side(r, q), side(r + 2, q)));
                         p[r].h[q] = K::fma(PC.c2, e, K::mul(PC.c1, f));
                         p[r].g[q] = STENCIL == 26 ? K::fma(PC.c3, e, K::mul(PC.c2, f)) : f;
                     }
@@ -921,7 +922,7 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
             const int oz = zc0 - 2 + i;   // output plane
 #pragma unroll
             for (int r = 0; r < RPT; ++r) {
-                if (gy + r >= g.ny || gx >= g.nx) continue;
+                if (r >= rows) continue;
                 T outv[VX];
                 // padded index of the row's first cell (32-bit, wraps): the cell's
                 // part of the stochastic-rounding hash
@@ -1015,10 +1016,10 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                                                K::mk(-C.dt * C.kmu, -C.dt * C.kmu));
                         } else {
                             const S *row = rbase + ((I + NS - 1) % NS) * STAGE + r * SW;
-                            P c[NP], w[NP], e[NP], u[NP], v[NP], d[NP];
-                            get_row<S, T, VX>(row, c, w, e);
-                            get_row<S, T, VX>(row - SW, u, d, d);
-                            get_row<S, T, VX>(row + SW, v, d, d);
+                            T x[VX + 2], n[VX], s[VX];
+                            get_row<S, T, VX>(row, x);
+                            Io<S, T>::lds(row - SW, n);
+                            Io<S, T>::lds(row + SW, s);
                             const T ep = C.eps;
                             const P s2 = K::mk(C.psi_grad, C.psi_grad);
                             auto diff = [&](P a, P b) {
@@ -1029,8 +1030,11 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
 #pragma unroll
                             for (int q = 0; q < NP; ++q) {
                                 const P sg = K::fma(PC.m2, z[r].c[q], PC.one);
-                                wl[q] = ti_local_w<T, STENCIL>(C, sg, K::mul(sg, sg), diff(e[q], w[q]),
-                                                               diff(v[q], u[q]), diff(p[r].c[q], m[r].c[q]));
+                                wl[q] = ti_local_w<T, STENCIL>(
+                                    C, sg, K::mul(sg, sg),
+                                    diff(K::mk(x[2 * q + 2], x[2 * q + 3]), K::mk(x[2 * q], x[2 * q + 1])),
+                                    diff(K::mk(s[2 * q], s[2 * q + 1]), K::mk(n[2 * q], n[2 * q + 1])),
+                                    diff(p[r].c[q], m[r].c[q]));
                             }
                         }
                     }
@@ -1063,8 +1067,8 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                         outv[2 * q + 1] = o.y;
                     }
                 }
-                S *optr = obase + (long long)oz * g.plane + (long long)r * g.pitch;
-                if (gx + VX <= g.nx) {
+                S *optr = out + r * g.pitch;
+                if (whole) {
                     Io<S, T>::st(optr, outv);
                     if (IMG && img) {
                         const int xo = ximg(), yo = yimg(r);
@@ -1087,6 +1091,7 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                 if (lane == 0) mbar_arrive(&empty[(I + NS - 1) % NS]);
             }
         }
+        if (i >= 2) out += g.plane;
         return i + 1 < nplanes;
     };
 
