@@ -245,6 +245,7 @@ void fill_stats_args(const spfm_grid *g, int flags, StatsArgs &a)
     for (int i = 0; i < 3; ++i) { a.n[i] = g->d.n[i]; a.ctr[i] = g->d.center[i]; }
     a.lambda = g->lambda;
     a.dx = g->dx;
+    a.band = band_const(a.n, a.ctr, a.lambda, a.dx);
     a.energy = (flags & SPFM_STATS_ENERGY) && g->scheme != SPFM_TI_LOCAL ? 1 : 0;
     a.scheme = g->scheme;
     a.stencil = g->stencil;

@@ -23,7 +23,6 @@
 // a step: sums 10.9 -> 6.0, correction and ghosts 67.1 + 3.4 -> 6.9 (one thread
 // added the 608 partials one by one); alpha formed once, by the last block of
 // the sums, was slower (9.1 + 5.1).
-#include "double_float.cuh"
 #include "spfm_internal.h"
 
 namespace spfm {

@@ -55,6 +55,18 @@ __device__ __forceinline__ DF df_mul_f(DF a, float b)
     const DF p = df_two_prod(a.hi, b);
     return df_fast_sum(p.hi, __fmaf_rn(a.lo, b, p.lo));
 }
+// a / b, b.hi not 0: the FP32 quotient and two corrections of its remainder
+__device__ __forceinline__ DF df_div(DF a, DF b)
+{
+    const float r = __fdividef(1.0f, b.hi);
+    const float q0 = __fmul_rn(a.hi, r);
+    const DF p = df_two_prod(q0, b.hi);
+    const float e0 = __fadd_rn(__fsub_rn(__fsub_rn(a.hi, p.hi), p.lo), __fmaf_rn(-q0, b.lo, a.lo));
+    const float q1 = __fmul_rn(e0, r);
+    const float e1 = __fmaf_rn(-q1, b.lo, __fmaf_rn(-q1, b.hi, e0));
+    const DF q = df_fast_sum(q0, q1);
+    return df_fast_sum(q.hi, __fmaf_rn(e1, r, q.lo));
+}
 __host__ __device__ __forceinline__ DF df_of(double x)
 {
     const float h = (float)x;

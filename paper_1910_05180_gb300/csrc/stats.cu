@@ -19,7 +19,6 @@
 
 #include <mutex>
 
-#include "double_float.cuh"
 #include "spfm_internal.h"
 
 namespace spfm {
@@ -94,34 +93,59 @@ __device__ __forceinline__ double potential(double phi, double a, double lam2_r2
     return lam2_r2 * (q + (1.0 - A) / (4.0 * A) * log((1.0 - A) / (1.0 - A * s * s)));
 }
 
-__device__ __forceinline__ void warp_reduce(double *v)
+// One block's (256 threads) partial from the sums of its threads.  An FP64
+// instruction of a warp holds the pipe 16 cycles for the whole SM, so the sums
+// are added 8 values a lane from shared memory before they are shuffled (13
+// instructions a sum, against 45 by shuffles in every warp), and the extrema
+// and the count stay out of FP64.
+template <class R>
+__device__ __forceinline__ R fewest(R a, R b) { return b < a ? b : a; }
+template <class R>
+__device__ __forceinline__ R most(R a, R b) { return b > a ? b : a; }
+constexpr int kSums = 5;   // volume, S_w, S_c, S_r, energy
+__device__ __forceinline__ int sum_slot(int s) { return s < 4 ? s : 7; }   // of a partial
+template <class R>
+__device__ __forceinline__ void block_reduce_store(const double (&sum)[kSums], R mn, R mx, double count, double *out)
 {
+    __shared__ double sm[kSums][256];
+    __shared__ R ext[2][8];
+    __shared__ double cnt[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int s = 0; s < kSums; ++s) sm[s][threadIdx.x] = sum[s];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int i = 0; i < kNStat; ++i) {
-            const double o = __shfl_down_sync(0xffffffffu, v[i], off);
-            if (i == 4) v[i] = fmin(v[i], o);
-            else if (i == 5) v[i] = fmax(v[i], o);
-            else v[i] += o;
-        }
+        mn = fewest(mn, __shfl_down_sync(0xffffffffu, mn, off));
+        mx = most(mx, __shfl_down_sync(0xffffffffu, mx, off));
     }
-}
-
-__device__ __forceinline__ void block_reduce_store(double *v, double *out)
-{
-    __shared__ double sm[32][kNStat];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    warp_reduce(v);
-    if (lane == 0)
-        for (int i = 0; i < kNStat; ++i) sm[warp][i] = v[i];
+    // counts are rare: a warp without one adds nothing
+    if (__any_sync(0xffffffffu, count != 0.0))
+        for (int off = 16; off > 0; off >>= 1) count += __shfl_down_sync(0xffffffffu, count, off);
+    if (lane == 0) {
+        ext[0][warp] = mn;
+        ext[1][warp] = mx;
+        cnt[warp] = count;
+    }
     __syncthreads();
-    if (warp == 0) {
-        for (int i = 0; i < kNStat; ++i)
-            v[i] = lane < nw ? sm[lane][i] : (i == 4 ? INFINITY : (i == 5 ? -INFINITY : 0.0));
-        warp_reduce(v);
-        if (lane == 0)
-            for (int i = 0; i < kNStat; ++i) out[i] = v[i];
+    if (warp < kSums) {
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) v += sm[warp][32 * w + lane];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+        if (lane == 0) out[sum_slot(warp)] = v;
+    } else if (warp == kSums && lane == 0) {
+        R lo = ext[0][0], hi = ext[1][0];
+        double n = cnt[0];
+        for (int w = 1; w < 8; ++w) {
+            lo = fewest(lo, ext[0][w]);
+            hi = most(hi, ext[1][w]);
+            n += cnt[w];
+        }
+        out[4] = (double)lo;
+        out[5] = (double)hi;
+        out[6] = n;
+        for (int i = 8; i < kNStat; ++i) out[i] = 0.0;
     }
 }
 
@@ -134,9 +158,14 @@ __device__ __forceinline__ void block_reduce_store(double *v, double *out)
 //     the band test run in the storage precision, where they are exact (the
 //     band limits 1e-6 and 1 - 1e-6 are not floats, so the first float above
 //     and the last float below them decide exactly the same cells);
-//   - an FP32 field's volume is summed per lane and row as an unevaluated pair
-//     (TwoSum, Knuth TAOCP vol. 2, 4.2.2), carried in 2^-48 fixed point;
-//   - band cells are queued per warp and evaluated 32 at a time, so the FP64
+//   - an FP32 field's volume is summed per lane and row as unevaluated pairs
+//     (TwoSum, Knuth TAOCP vol. 2, 4.2.2), two chains on the paired FP32
+//     instructions, carried in 2^-48 fixed point;
+//   - a row of cells is taken as finite and tested for band cells as a whole (a
+//     sum that is not finite has the lane look at its cells one by one; one
+//     minimum of |phi - 1/2| over 16 cells says whether any may lie in the band),
+//     so the cells of the bulk phases cost about 6 instructions each;
+//   - band cells are queued per warp and evaluated 32 at a time, so the
 //     inversion of the profile runs with every lane busy.
 template <class S> struct Scr { using T = float; };
 template <> struct Scr<double> { using T = double; };
@@ -173,6 +202,21 @@ template <> struct Row16<double> {
     }
 };
 
+// cell k of the storage elements in the words u
+template <class S> __device__ __forceinline__ typename Scr<S>::T word_cell(const unsigned *u, int k);
+template <> __device__ __forceinline__ float word_cell<float>(const unsigned *u, int k)
+{
+    return __uint_as_float(u[k]);
+}
+template <> __device__ __forceinline__ float word_cell<__nv_bfloat16>(const unsigned *u, int k)
+{
+    return __uint_as_float((k & 1) ? (u[k / 2] & 0xffff0000u) : (u[k / 2] << 16));
+}
+template <> __device__ __forceinline__ double word_cell<double>(const unsigned *u, int k)
+{
+    return __hiloint2double((int)u[2 * k + 1], (int)u[2 * k]);
+}
+
 // 1e-6 < x < 1 - 1e-6 for an FP32 x: the limits are not FP32 numbers, so the
 // test compares with the first float above 1e-6 and the last float below
 // 1 - 1e-6 (written out: a rounding conversion here would run on the FP64 pipe
@@ -182,6 +226,19 @@ __device__ __forceinline__ bool in_band(float x)
     return x >= 0x1.0c6f7cp-20f && x <= 0x1.ffffdep-1f;
 }
 __device__ __forceinline__ bool in_band(double x) { return x > 1e-6 && x < 1.0 - 1e-6; }
+
+// the upper words of 1e-6 and 1 - 1e-6 bound those of the band's cells
+static_assert(0x3eb0c6f7u < 0x3feffffeu, "band limits");
+// a double's bits as a signed integer of the same order (-0 below +0), and back
+__device__ __forceinline__ long long order_key(double x)
+{
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double key_value(long long k)
+{
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
+}
 
 // y * 2^48 truncated toward zero, for |y| < 2^14 (the bits below 2^-48 drop)
 __device__ __forceinline__ long long fix48(float y)
@@ -201,21 +258,35 @@ __device__ __forceinline__ long long fix48(float y)
 // point could overflow.
 template <class R> struct VolSum;
 template <> struct VolSum<float> {
-    float s = 0.0f, c = 0.0f;
+    float2 s = {0.0f, 0.0f}, c = {0.0f, 0.0f};   // two chains
     long long fix = 0;
     double sum = 0.0;
     int rows = 0;
-    __device__ __forceinline__ void add(float x)
+    static __device__ __forceinline__ float2 sub(float2 a, float2 b)
     {
-        const float t = s + x, z = t - s;
-        c += (s - (t - z)) + (x - z);
+        return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
+    }
+    __device__ __forceinline__ void add(float2 x)
+    {
+        const float2 t = __fadd2_rn(s, x), z = sub(t, s);
+        c = __fadd2_rn(c, __fadd2_rn(sub(s, sub(t, z)), sub(x, z)));
         s = t;
+    }
+    __device__ __forceinline__ void add(float x) { add(make_float2(x, 0.0f)); }
+    __device__ __forceinline__ bool finite() const { return isfinite(s.x) && isfinite(s.y); }
+    __device__ __forceinline__ float4 row() const { return make_float4(s.x, s.y, c.x, c.y); }
+    __device__ __forceinline__ void set_row(float4 r)
+    {
+        s = make_float2(r.x, r.y);
+        c = make_float2(r.z, r.w);
     }
     __device__ __forceinline__ void end_row()
     {
-        if (fabsf(s) < 256.0f) fix += fix48(s) + fix48(c);
-        else sum += (double)s + (double)c;
-        s = c = 0.0f;
+        const DF t = df_two_sum(s.x, s.y);
+        const float lo = (c.x + c.y) + t.lo;
+        if (fabsf(t.hi) < 256.0f) fix += fix48(t.hi) + fix48(lo);
+        else sum += (double)t.hi + (double)lo;
+        set_row(make_float4(0.0f, 0.0f, 0.0f, 0.0f));
         if (++rows == 64) {
             sum += (double)fix * 0x1p-48;
             fix = 0;
@@ -227,6 +298,7 @@ template <> struct VolSum<float> {
 template <> struct VolSum<double> {
     double sum = 0.0;
     __device__ __forceinline__ void add(double x) { sum += x; }
+    __device__ __forceinline__ int row() const { return 0; }
     __device__ __forceinline__ void end_row() {}
     __device__ __forceinline__ double total() const { return sum; }
 };
@@ -248,7 +320,7 @@ __global__ void ln_table_kernel()
     }
 }
 
-// ln y for y = hi + lo in [2^-126, 1], table-driven (Tang, ACM TOMS 16, 1990):
+// ln y for y = hi + lo in [2^-63, 2^63], table-driven (Tang, ACM TOMS 16, 1990):
 // hi = 2^k m, m in [1, 2); F = 1 + j/256 takes the top 8 fraction bits of m, so
 // f = (m - F) + lo 2^-k holds y 2^-k - F to double-float accuracy and u = f/F
 // lies in (-2^-24, 2^-8).  ln(1 + u) is its Taylor series: u - u^2/2 in
@@ -286,11 +358,9 @@ template <class R> struct BandCell {
 };
 
 // Sec. 2.3 sums of one band cell, in double-float: q = phi(1 - phi),
-// psi = (lambda/2) artanh(1 - 2 phi) = (lambda/4) (ln(1 - phi) - ln phi),
-// p = dx (i, j, k).  Absolute error of psi below about 1e-13.
-struct BandConst {
-    DF dxn0, dxn1, dxn2, dx, neg_c0, neg_c1, neg_c2, quarter_lambda;
-};
+// psi = (lambda/2) artanh(1 - 2 phi) = (lambda/4) ln((1 - phi) / phi), one
+// logarithm of a double-float quotient, p = dx (i, j, k).  Absolute error of psi
+// below about 1e-13.
 template <class R> struct BandPhi;
 template <> struct BandPhi<float> {   // FP32 and BF16 storage: phi exact, 1 - phi exact as a pair
     static __device__ __forceinline__ void get(float x, DF &ph, DF &om)
@@ -316,10 +386,9 @@ __device__ __forceinline__ void band_cell(const BandConst &bc, const BandCell<R>
     DF ph, om;
     BandPhi<R>::get(c.phi, ph, om);
     const DF q = df_mul(ph, om);
-    const LnParts l1 = ln_parts(om, tab), l0 = ln_parts(ph, tab);
-    const float2 kl = kln2[l1.k - l0.k + 64];
-    DF d = df_add(DF{kl.x, kl.y}, df_add(l1.lnF, df_neg(l0.lnF)));
-    d = df_add(d, df_add(l1.s, df_neg(l0.s)));
+    const LnParts l = ln_parts(df_div(om, ph), tab);
+    const float2 kl = kln2[l.k + 64];
+    const DF d = df_add(df_add(DF{kl.x, kl.y}, l.lnF), l.s);
     const DF psi = df_mul(bc.quarter_lambda, d);
     const DF fi = df_of_int(c.i);
     const DF pn = df_add(c.pn_row, df_mul(bc.dxn0, fi));
@@ -354,13 +423,10 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
     const float4 *tab = g_ln_tab;
     const float2 *kln2 = g_kln2;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double v[kNStat];
-#pragma unroll
-    for (int i = 0; i < kNStat; ++i) v[i] = 0.0;
     R mn = R(INFINITY), mx = R(-INFINITY);
+    long long klo = order_key(INFINITY), khi = order_key(-INFINITY);   // FP64 extrema as order keys
     int nonfinite = 0;
-    const BandConst bconst = {df_of(a.dx * a.n[0]), df_of(a.dx * a.n[1]), df_of(a.dx * a.n[2]), df_of(a.dx),
-                              df_of(-a.ctr[0]),      df_of(-a.ctr[1]),      df_of(-a.ctr[2]), df_of(0.25 * a.lambda)};
+    const BandConst &bconst = a.band;
     BandSums sums;
     int head = 0, tail = 0, band_rows = 0;   // ring positions and band rows so far (warp-uniform)
     // evaluate the waiting cell at ring position q (this lane's)
@@ -376,7 +442,7 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
     };
     VolSum<R> vol;
     const long long rows = (long long)a.g.ny * a.g.nz;
-    const int nvec = (a.g.nx + E - 1) / E;
+    const int nvec = (a.g.nx + E - 1) / E, nwhole = a.g.nx / E;   // 16-byte pieces of a row, and whole ones
     // rows (j, k) dealt round-robin to the warps; ny nz < 2^30, and (j, k)
     // advance by the stride's split so that no row divides (64-bit division
     // is emulated in FP64, the slow pipe of this GPU)
@@ -389,28 +455,96 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
         const uint4 *src = (const uint4 *)(f + cell_index(a.g, 0, j, k));
         for (int v0 = 0; v0 < nvec; v0 += 32 * V) {
             uint4 w[V];
+            const auto before = vol.row();
 #pragma unroll
             for (int t = 0; t < V; ++t) {
                 const int vi = v0 + 32 * t + lane;
                 w[t] = vi < nvec ? __ldg(src + vi) : make_uint4(0u, 0u, 0u, 0u);
             }
+            // extrema and volume of the lane's whole pieces (a piece that a row's
+            // end cuts goes cell by cell), and whether any cell may lie in the band
+            bool near = false;
+            R lo = R(INFINITY), hi = R(-INFINITY);
+            if constexpr (sizeof(R) == 4) {
+                float far = 1.0f;   // the least |phi - 1/2|
+#pragma unroll
+                for (int t = 0; t < V; ++t) {
+                    const int vi = v0 + 32 * t + lane;
+                    if (vi < nwhole) {
+#pragma unroll
+                        for (int e = 0; e < E; e += 2) {
+                            const float2 x = make_float2(Row16<S>::get(w[t], e), Row16<S>::get(w[t], e + 1));
+                            vol.add(x);
+                            lo = fminf(fminf(lo, x.x), x.y);
+                            hi = fmaxf(fmaxf(hi, x.x), x.y);
+                            const float2 d = __fadd2_rn(x, make_float2(-0.5f, -0.5f));
+                            far = fminf(fminf(far, fabsf(d.x)), fabsf(d.y));
+                        }
+                    } else if (vi < nvec) {
+#pragma unroll
+                        for (int e = 0; e < E; ++e)
+                            if (vi * E + e < a.g.nx) {
+                                const float x = Row16<S>::get(w[t], e);
+                                near = near || in_band(x);
+                                vol.add(x);
+                                lo = fminf(lo, x);
+                                hi = fmaxf(hi, x);
+                            }
+                    }
+                }
+                near = near || far < 0.5f - 0.5e-6f;   // band cells have |phi - 1/2| < 1/2 - 1e-6
+                if (!vol.finite()) {   // the sweep again, without the cells that are not
+                    vol.set_row(before);
+                    lo = R(INFINITY);
+                    hi = R(-INFINITY);
+#pragma unroll
+                    for (int t = 0; t < V; ++t)
+#pragma unroll
+                        for (int e = 0; e < E; ++e)
+                            if ((v0 + 32 * t + lane) * E + e < a.g.nx) {
+                                const float x = Row16<S>::get(w[t], e);
+                                if (!isfinite(x)) {
+                                    ++nonfinite;
+                                    continue;
+                                }
+                                vol.add(x);
+                                lo = fminf(lo, x);
+                                hi = fmaxf(hi, x);
+                            }
+                }
+            } else {
+                // FP64 cells: the one FP64 instruction each is the volume's add; the
+                // rest compares integers (upper words for the tests)
+#pragma unroll
+                for (int t = 0; t < V; ++t)
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if ((v0 + 32 * t + lane) * E + e < a.g.nx) {
+                            const R x = Row16<S>::get(w[t], e);
+                            const unsigned h = (unsigned)__double2hiint(x);
+                            if ((h & 0x7ff00000u) == 0x7ff00000u) {
+                                ++nonfinite;
+                                continue;
+                            }
+                            vol.add(x);
+                            const long long k = order_key(x);
+                            klo = k < klo ? k : klo;
+                            khi = k > khi ? k : khi;
+                            near = near || h - 0x3eb0c6f7u <= 0x3feffffeu - 0x3eb0c6f7u;
+                        }
+            }
+            if constexpr (sizeof(R) == 4) {
+                mn = fewest(mn, lo);
+                mx = most(mx, hi);
+            }
+            if (!__any_sync(0xffffffffu, near)) continue;
             unsigned bm = 0u;   // band cells of this lane among its E * V
 #pragma unroll
             for (int t = 0; t < V; ++t)
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
-                    const int i = (v0 + 32 * t + lane) * E + e;
                     const R x = Row16<S>::get(w[t], e);
-                    if (i < a.g.nx) {
-                        if (!isfinite(x)) {
-                            ++nonfinite;
-                        } else {
-                            vol.add(x);
-                            mn = x < mn ? x : mn;
-                            mx = x > mx ? x : mx;
-                            if (in_band(x)) bm |= 1u << (t * E + e);
-                        }
-                    }
+                    if (in_band(x) && (v0 + 32 * t + lane) * E + e < a.g.nx) bm |= 1u << (t * E + e);
                 }
             if (__any_sync(0xffffffffu, bm != 0u)) {
                 if (!row_known) {
@@ -426,48 +560,58 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
                     }
                     row_known = true;
                 }
-                // queue the sweep's band cells in four parts (a warp prefix sum
-                // places each lane's cells), evaluating full warps after each
+                // Queue the sweep's band cells in four parts of 4 cells a lane (a warp
+                // prefix sum places each lane's), evaluating full warps after each.
+                // The parts stay a loop, the sweep's words moving down by one part a
+                // round: unrolled, four copies of the evaluation did not fit the
+                // instruction cache (no_instruction the top stall).
+                constexpr int kW = (int)sizeof(S);   // 32-bit words of 4 cells
+                unsigned u[4 * V];
 #pragma unroll
+                for (int t = 0; t < V; ++t) {
+                    u[4 * t] = w[t].x;
+                    u[4 * t + 1] = w[t].y;
+                    u[4 * t + 2] = w[t].z;
+                    u[4 * t + 3] = w[t].w;
+                }
+#pragma unroll 1
                 for (int part = 0; part < 4; ++part) {
-                    const unsigned m = (bm >> (4 * part)) & 0xfu;
-                    const int c = __popc(m);
-                    int incl = c;
+                    const unsigned m = bm & 0xfu;
+                    if (__any_sync(0xffffffffu, m != 0u)) {
+                        const int c = __popc(m);
+                        int incl = c;
 #pragma unroll
-                    for (int d = 1; d < 32; d <<= 1) {
-                        const int y = __shfl_up_sync(0xffffffffu, incl, d);
-                        if (lane >= d) incl += y;
-                    }
-                    int pos = tail + incl - c;
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        constexpr int kE = E;
-                        const int b = 4 * part + u;
-                        if (m & (1u << u)) {
-                            const int r = pos & (kRing - 1);
-                            ring_phi[warp][r] = Row16<S>::get(w[b / kE], b % kE);
-                            ring_i[warp][r] = (v0 + 32 * (b / kE) + lane) * kE + b % kE;
-                            ring_slot[warp][r] = (unsigned char)slot;
-                            ++pos;
+                        for (int d = 1; d < 32; d <<= 1) {
+                            const int y = __shfl_up_sync(0xffffffffu, incl, d);
+                            if (lane >= d) incl += y;
                         }
+                        int pos = tail + incl - c;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            if (m & (1u << k)) {
+                                const int r = pos & (kRing - 1);
+                                const int b = 4 * part + k;   // cell of the lane's E * V
+                                ring_phi[warp][r] = word_cell<S>(u, k);
+                                ring_i[warp][r] = (v0 + 32 * (b / E) + lane) * E + b % E;
+                                ring_slot[warp][r] = (unsigned char)slot;
+                                ++pos;
+                            }
+                        }
+                        tail += __shfl_sync(0xffffffffu, incl, 31);
+                        __syncwarp();
+                        for (; tail - head >= 32; head += 32) eval_at(head + lane);
+                        __syncwarp();   // reads of evaluated cells before the next part's writes
                     }
-                    tail += __shfl_sync(0xffffffffu, incl, 31);
-                    __syncwarp();
-                    for (; tail - head >= 32; head += 32) eval_at(head + lane);
-                    __syncwarp();   // reads of evaluated cells before the next part's writes
+                    bm >>= 4;
+#pragma unroll
+                    for (int k = 0; k + kW < 4 * V; ++k) u[k] = u[k + kW];
                 }
             }
         }
         vol.end_row();
     }
-    v[0] = vol.total();
     if (lane < tail - head) eval_at(head + lane);
-    v[1] = df_to_double(sums.w);
-    v[2] = df_to_double(sums.c);
-    v[3] = df_to_double(sums.r);
-    v[4] = (double)mn;
-    v[5] = (double)mx;
-    v[6] = (double)nonfinite;
+    double energy = 0.0;
     if (a.energy) {   // Eq. 1 at dF = 0, one cell per thread, contiguous rows per block
         const long long r0 = blk * rows / nblk, r1 = (blk + 1) * rows / nblk;
         const double e_pref = a.Gamma / (a.C_gamma * a.lambda);
@@ -487,23 +631,31 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
                     e += a.w[kk] * (0.5 * a.lambda * a.lambda * dp * dp / r2 +
                                     potential(ph, a.a[kk], a.lambda * a.lambda / r2, is_fd_scheme(a.scheme)));
                 }
-                v[7] += e_pref * e;
+                energy += e_pref * e;
             }
         }
     }
-    block_reduce_store(v, partial_out);
+    const double total[kSums] = {vol.total(), df_to_double(sums.w), df_to_double(sums.c), df_to_double(sums.r),
+                                 energy};
+    if constexpr (sizeof(R) == 8) {
+        mn = (R)key_value(klo);
+        mx = (R)key_value(khi);
+    }
+    block_reduce_store<R>(total, mn, mx, (double)nonfinite, partial_out);
 }
 
 template <class S>
-__global__ void __launch_bounds__(256) stats_kernel(const StatsArgs a, const S *f, double *partials)
+__global__ void __launch_bounds__(256, sizeof(S) == 8 ? 2 : 3) stats_kernel(const StatsArgs a, const S *f, double *partials)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     stats_pass<S>(a, f, partials + (long long)blockIdx.x * kNStat, blockIdx.x, gridDim.x);
 }
 
 // blockIdx.y selects the grid of the batch
 template <class S>
-__global__ void __launch_bounds__(256) stats_batch_kernel(const StatsJob *jobs, double *partials)
+__global__ void __launch_bounds__(256, 2) stats_batch_kernel(const StatsJob *jobs, double *partials)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const StatsJob &j = jobs[blockIdx.y];
     stats_pass<S>(j.a, (const S *)j.field[j.cur],
                   partials + ((long long)blockIdx.y * kBatchStatsBlocks + blockIdx.x) * kNStat,
@@ -513,23 +665,19 @@ __global__ void __launch_bounds__(256) stats_batch_kernel(const StatsJob *jobs, 
 // blockIdx.x selects a grid: reduce its nblocks partials into out[blockIdx.x]
 __global__ void __launch_bounds__(256) stats_final_kernel(const double *partials, int nblocks, double *out)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // launched while the pass runs
     partials += (long long)blockIdx.x * nblocks * kNStat;
     out += (long long)blockIdx.x * kNStat;
-    double v[kNStat];
-#pragma unroll
-    for (int i = 0; i < kNStat; ++i) v[i] = 0.0;
-    v[4] = INFINITY;
-    v[5] = -INFINITY;
+    double sum[kSums] = {0.0, 0.0, 0.0, 0.0, 0.0}, mn = INFINITY, mx = -INFINITY, count = 0.0;
     for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
+        const double *p = partials + (long long)b * kNStat;
 #pragma unroll
-        for (int i = 0; i < kNStat; ++i) {
-            const double x = partials[(long long)b * kNStat + i];
-            if (i == 4) v[i] = fmin(v[i], x);
-            else if (i == 5) v[i] = fmax(v[i], x);
-            else v[i] += x;
-        }
+        for (int s = 0; s < kSums; ++s) sum[s] += p[sum_slot(s)];
+        mn = fmin(mn, p[4]);
+        mx = fmax(mx, p[5]);
+        count += p[6];
     }
-    block_reduce_store(v, out);
+    block_reduce_store<double>(sum, mn, mx, count, out);
 }
 
 size_t stats_scratch_bytes()
@@ -586,6 +734,21 @@ template <class S> static int stats_blocks()
     return cached[dev];
 }
 
+// the reduction of n grids' partials, which may launch while the pass before it runs
+static cudaError_t launch_final(int n, const double *partials, int nblocks, double *out, cudaStream_t st)
+{
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(n);
+    lc.blockDim = dim3(256);
+    lc.stream = st;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, stats_final_kernel, partials, nblocks, out);
+}
+
 cudaError_t launch_stats(const StatsArgs &a, const void *field, double *partials, double *final_out,
                          cudaStream_t st)
 {
@@ -604,8 +767,7 @@ cudaError_t launch_stats(const StatsArgs &a, const void *field, double *partials
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    stats_final_kernel<<<1, 256, 0, st>>>(partials, nb, final_out);
-    return cudaGetLastError();
+    return launch_final(1, partials, nb, final_out, st);
 }
 
 cudaError_t launch_stats_batch(const StatsJob *jobs, int n, int dtype, double *partials, double *finals,
@@ -620,8 +782,7 @@ cudaError_t launch_stats_batch(const StatsJob *jobs, int n, int dtype, double *p
     else stats_batch_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(jobs, partials);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    stats_final_kernel<<<n, 256, 0, st>>>(partials, kBatchStatsBlocks, finals);
-    return cudaGetLastError();
+    return launch_final(n, partials, kBatchStatsBlocks, finals, st);
 }
 
 }  // namespace spfm
