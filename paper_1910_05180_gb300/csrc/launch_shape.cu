@@ -25,6 +25,11 @@
 //   SM, which holds for the streaming kernels at three or four CTAs per SM;
 //   kernels with fewer keep the rule of many rounds.
 //
+// - Less than a round at 4 planes: the shortest chunks that still fit one round,
+//   since such a launch lasts as long as one CTA's march (FP32, contact faces, 13
+//   groups, us a step: 32^3 4 planes 7.6, 1 (chosen) 5.2; 64^3 7.6 and 5.4; 96^3
+//   4 planes 8.0, 3 (chosen) 7.6, 2 (more than a round) 9.9).
+//
 // TI_n has a rule of its own: its CTAs differ in work (those in the interface
 // band compute the 13 couplings of each cell, a plane of them some 2 us; those
 // in the bulk do not), so it wants many small CTAs.  About six rounds of
@@ -36,14 +41,14 @@
 // 256^3 16: 96.0, 8: 90.4 (9 chosen), 4: 94.2; 320^3 16 (chosen): 124.6, 8: 129.
 //
 // The FP64 kernels (CF and TI global) are bound by the FP64 pipe, which the CTAs
-// of an SM share: what counts is the work of the fullest SM, n CTAs on each of
-// at most ceil(CTAs / SMs), a plane of a CTA costing about 9 FP64 instructions a
-// cell as it is read and 18 more as it is written (the halo planes are only
-// read).  One CTA alone keeps the pipe about a third busy, so one or two on an
-// SM take as long as three.  Chunks of 1 to 64 planes, the least work, ties to
-// the longer chunk.  Measured, us a step (planes per CTA): 128 x 32 x 32 7-point
-// 1 (chosen) 16.4, 2: 18.4, 4 (the streaming rule): 18.8; 48^3 1 (chosen) 51.0,
-// 4: 79.2; 96^3 4 (chosen) 110, 2: 125, 12: 264; 256^3 37 (chosen) 1038, 16: 1066.
+// of an SM share: what counts is the work of the fullest SM, ceil(CTAs / SMs)
+// CTAs, a plane of a CTA costing about 9 FP64 instructions a cell as it is read
+// and 18 more as it is written (the halo planes are only read).  A CTA alone on
+// its SM leaves the pipe idle a fifth of the time, two leave it 2 %.  Chunks of
+// 1 to 64 planes, the least work, ties to the longer chunk.  Measured, us a step
+// (planes per CTA): 128 x 32 x 32 7-point 2 (chosen) 10.6, 1: 15.0, 4 (the
+// streaming rule) 15.8; 72^3 4 (chosen) 81, 2: 100; 96^3 6 (chosen) 107, 12: 126,
+// 2: 125; 100^3 10 (chosen) 167, 5: 225; 256^3 37 (chosen) 1047, 16: 1066.
 #include <map>
 #include <mutex>
 #include <queue>
@@ -106,13 +111,17 @@ static int model_zchunk(int tiles, int nz, int per_sm, int slots, int target)
     return best;
 }
 
+// the shortest chunks whose CTAs fit one round
+static int one_round_zchunk(int tiles, int nz, int slots)
+{
+    const int chunks = slots / tiles < nz ? slots / tiles : nz;
+    return (nz + chunks - 1) / chunks;
+}
+
 // planes per CTA of a TI_n launch (see above)
 static int uneven_zchunk(int tiles, int nz, int slots)
 {
-    if ((long long)tiles * ((nz + 3) / 4) < slots) {
-        const int chunks = slots / tiles < nz ? slots / tiles : nz;
-        return (nz + chunks - 1) / chunks;
-    }
+    if ((long long)tiles * ((nz + 3) / 4) < slots) return one_round_zchunk(tiles, nz, slots);
     const long long zc = ((long long)tiles * nz + 6LL * slots - 1) / (6LL * slots);
     return zc < 4 ? 4 : (zc > 16 ? 16 : (int)zc);
 }
@@ -124,7 +133,8 @@ static int fp64_zchunk(int tiles, int nz, int sms)
     long long best_work = -1;
     for (int zc = 1; zc <= (nz < 64 ? nz : 64); ++zc) {
         const long long ctas = (long long)tiles * ((nz + zc - 1) / zc);
-        const long long n = (ctas + sms - 1) / sms, work = (n < 3 ? 3 : n) * (9 * (zc + 2) + 18 * zc);
+        const long long n = (ctas + sms - 1) / sms, idle = n == 1 ? 20 : (n == 2 ? 2 : 0);
+        const long long work = n * (100 + idle) * (9 * (zc + 2) + 18 * zc);
         if (best_work < 0 || work <= best_work) {
             best_work = work;
             best = zc;
@@ -166,7 +176,8 @@ int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target, in
     if (g_zc.size() >= 4096) g_zc.clear();   // many grid shapes (a serving process): start over
     const int zc = family == kUneven ? uneven_zchunk(tiles, nz, slots)
                    : family == kFp64 ? fp64_zchunk(tiles, nz, sms)
-                                     : model_zchunk(tiles, nz, per_sm, slots, target);
+                   : (long long)tiles * ((nz + 3) / 4) <= slots ? one_round_zchunk(tiles, nz, slots)
+                                                                : model_zchunk(tiles, nz, per_sm, slots, target);
     g_zc[zk] = zc;
     return zc;
 }
