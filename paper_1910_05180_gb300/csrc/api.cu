@@ -516,10 +516,7 @@ spfm_status spfm_step(spfm_grid *g, int n_steps, double M, double Gamma, double 
     const bool face_kernel = !images && !inline_faces;
     const int skip = g->skip_copy && n_steps > 0 ? kSkipCopy : 0;
     g->skip_copy = g->skip_copy && n_steps == 0;
-    auto mode_of = [&](int i) {
-        const int m = images ? kWaitAll | kImages : (inline_faces ? kWaitAll | kEarly : (i == 0 ? kWaitAll : kWaitFaces));
-        return m | (i == 0 ? skip : 0);
-    };
+    auto mode_of = [&](int i) { return (images ? kImages : 0) | (i == 0 ? skip : 0); };
     int *err = err_word(g);
     if (g->d.dtype == SPFM_F64) {
         StepCoef<double> c;
@@ -531,7 +528,7 @@ spfm_status spfm_step(spfm_grid *g, int n_steps, double M, double Gamma, double 
                                             (double *)g->d.field[1 - g->cur], err, cfg, &g->tma,
                                             g->cur, s);
             if (e == cudaSuccess && face_kernel)
-                e = launch_fill_ghosts(g->geom, g->d.dtype, m.aface, g->d.field[1 - g->cur], s, 1);
+                e = launch_fill_ghosts(g->geom, g->d.dtype, m.aface, g->d.field[1 - g->cur], s, 1, true);
             if (e != cudaSuccess) return cuda_fail(g, e, "spfm_step");
             g->cur ^= 1;
         }
@@ -553,7 +550,7 @@ spfm_status spfm_step(spfm_grid *g, int n_steps, double M, double Gamma, double 
                                      (__nv_bfloat16 *)g->d.field[1 - g->cur], err, cfg, &g->tma,
                                      g->cur, s);
             if (e == cudaSuccess && face_kernel)
-                e = launch_fill_ghosts(g->geom, g->d.dtype, m.aface, g->d.field[1 - g->cur], s, 1);
+                e = launch_fill_ghosts(g->geom, g->d.dtype, m.aface, g->d.field[1 - g->cur], s, 1, true);
             if (e != cudaSuccess) return cuda_fail(g, e, "spfm_step");
             g->cur ^= 1;
         }
@@ -604,7 +601,7 @@ spfm_status spfm_step_conserving(spfm_grid *g, int n_steps, double M, double Gam
     }
     for (int i = 0; i < n_steps; ++i) {
         void *src = g->d.field[g->cur], *dst = g->d.field[1 - g->cur];
-        cfg.mode = kWaitAll | kEarly;   // the sums and the correction wait for their predecessor, too
+        cfg.mode = 0;
         cf.sr_key = sr_step_key(g->sr_seed, g->steps + i);
         cudaError_t e;
         if (g->d.dtype == SPFM_F64)

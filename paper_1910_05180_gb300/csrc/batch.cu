@@ -125,6 +125,7 @@ struct spfm_batch {
     std::vector<spfm_grid *> grids;
     int n = 0, dtype = 0, depth = 0, policy = SPFM_TILES_FIT;
     int ctas[2] = {0, 0};     // CTAs of each shape's launch
+    int slots = 0;            // resident CTAs of the device
     int nitems0 = 0;          // items of shape 0; the shape-1 items follow them in the list
     char *scratch = nullptr;
     cudaStream_t stream = nullptr;
@@ -220,7 +221,7 @@ static cudaError_t set_depth(spfm_batch *b, int depth)
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int slots = sms * kBatchCtasPerSm;
+    const int slots = b->slots = sms * kBatchCtasPerSm;
     Deal d;
     if (depth == 0) {
         long long best = -1;
@@ -267,7 +268,8 @@ static cudaError_t launch_shape(spfm_batch *b, int shape, int parity, int stenci
     int *err = (int *)(b->scratch + b->L.err);
     const long long *steps = (const long long *)(b->scratch + b->L.steps);
     const BatchList list = {(const BatchItem *)(b->scratch + b->L.items) + (shape ? b->nitems0 : 0),
-                            (const int *)(b->scratch + b->L.starts) + shape * (kMaxCtas + 1), b->ctas[shape]};
+                            (const int *)(b->scratch + b->L.starts) + shape * (kMaxCtas + 1), b->ctas[shape],
+                            b->ctas[shape] >= b->slots};
     const int fwd = b->inline_faces ? 1 : 0;
     const cudaStream_t st = b->stream;
     if (b->dtype == SPFM_F64) return launch_batch_f64(grids, list, parity, err, stencil, kind, st, fwd);

@@ -112,7 +112,7 @@ template <class S>
 __global__ void __launch_bounds__(32 * kWarps) conserve_sums_kernel(const GridGeom g, const S *src, const S *dst,
                                                                     double *partials)
 {
-    asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     using T = typename Cell<S>::T;
     constexpr int E = Vec<S>::E;
     const int lane = threadIdx.x & 31;
@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(32 * kWarps) conserve_sums_kernel(const GridGe
     block_sum2(dsum, qsum);
     if (threadIdx.x == 0) partials[2 * blockIdx.x] = dsum;
     if (threadIdx.x == 32) partials[2 * blockIdx.x + 1] = dsum;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Boundary kinds of the faces as bits (an axis is periodic on both faces or on
@@ -223,7 +224,7 @@ __global__ void __launch_bounds__(32 * kWarps)
     conserve_apply_kernel(const GridGeom g, const __grid_constant__ Faces<typename Cell<S>::T> fc, const S *src,
                           S *dst, const double *partials, double *alpha_out)
 {
-    asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     constexpr int E = Vec<S>::E;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rows = g.ny * g.nz;
@@ -264,6 +265,7 @@ __global__ void __launch_bounds__(32 * kWarps)
             write_cells<S, CONTACT, E>(g, fc, dst, d, i, j, k);
         }
     }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <class S>

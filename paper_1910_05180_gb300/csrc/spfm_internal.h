@@ -185,7 +185,7 @@ __device__ inline double contact_shift_rn(double v, double a)
 struct LaunchCfg {
     int stencil;   // 6, 18, 26
     int scheme;    // SPFM_TI_GLOBAL, SPFM_TI_LOCAL, SPFM_FD
-    int mode;      // kWaitFaces | kWaitAll | kImages
+    int mode;      // a set of the bits below
     int rounding = SPFM_ROUND_NEAREST;   // SPFM_ROUND_STOCHASTIC: the *_sr kernels
     int zchunk = 0;   // planes per CTA; 0: pick_zchunk
     int *zchunk_used = nullptr;   // receives the planes per CTA of the launch (host, optional)
@@ -199,18 +199,20 @@ struct LaunchCfg {
 enum { kStream = 0, kUneven = 1, kFp64 = 2 };
 int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target, int family);
 
-// How a step launch sits in the stream (programmatic dependent launch):
-//   kWaitFaces  the previous kernel refreshes src's ghosts: boxes touching a face wait for it
-//   kWaitAll    every box waits for the previous kernel
+// How a step launch runs.  Launches chain by programmatic dependent launch: every
+// kernel of a call may start while the one before runs and waits for the whole of
+// it before it reads.  When a kernel lets the next one start matters for balance:
+// CTAs that arrive early take the slots that happen to be free and crowd some
+// SMs, so a launch of few rounds does so at its end (us a step, start -> end:
+// 64^3 periodic TI_<111> 4.2 -> 3.3, 150 x 133 x 117 contact 11.3 -> 10.7, 64^3 FP64
+// 38.0 -> 24.7), while many rounds (kEarly) fill the slots that their tail leaves
+// (320^3 TI_n 155.3 -> 154.1).
 //   kImages     all faces periodic: the step writes the ghost images of its new cells
-//               itself (no face kernel follows) and lets the next step launch early
+//               itself (no face kernel follows)
 //   kSkipCopy   test of the bounded waits: the first CTA skips one plane's copy
 //               (spfm_debug_skip_copy), its waits give up and set the error word
-//   kEarly      the kernel that follows waits for the whole of this one itself (the
-//               next step, where the step computes the ghosts of non-periodic faces as
-//               it reads them; the constant-volume sums): the step lets it launch at
-//               its start, like the image-writing kernels
-constexpr int kWaitFaces = 1, kWaitAll = 2, kImages = 4, kSkipCopy = 8, kEarly = 16;
+//   kEarly      the next kernel may launch at this one's start (set by the launch)
+constexpr int kImages = 4, kSkipCopy = 8, kEarly = 16;
 
 // TMA tensor maps of a grid's two field buffers, encoded on first use (tma.cu).
 struct TmaCache {
@@ -279,9 +281,11 @@ cudaError_t launch_conserve(const GridGeom &g, int dtype, const double aface[6],
 cudaError_t launch_shift_x(const GridGeom &g, int dtype, const void *src, void *dst, int cells, cudaStream_t st);
 
 // Ghost layer of a buffer from its interior: all faces (x_faces = 1) or the y
-// and z faces only.  Face sizes must stay below 2^31 cells.
+// and z faces only.  Face sizes must stay below 2^31 cells.  chained: the kernel
+// may launch while the one before it runs (it waits for it); the next kernel
+// must then wait for all of this one.
 cudaError_t launch_fill_ghosts(const GridGeom &g, int dtype, const double aface[6], void *field,
-                               cudaStream_t st, int x_faces);
+                               cudaStream_t st, int x_faces, bool chained = false);
 
 // Constants of the band sums as double-float pairs, formed on the host (formed
 // in the kernel they cost an evaluation of 32 cells some 20 FP64 instructions):
@@ -331,6 +335,7 @@ struct BatchList {
     const BatchItem *work;
     const int *start;
     int ctas;
+    int early;   // the CTAs fill every slot: the next step's may launch at once
 };
 constexpr int kBatchCtasPerSm = 3;   // resident CTAs of the batch kernels (four: 96 registers, spills, 6-11 % slower)
 

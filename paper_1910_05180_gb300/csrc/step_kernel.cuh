@@ -15,14 +15,14 @@
 //
 // Boundary conditions.  The kernel reads the ghost layer.  In general it
 // writes interior cells only and a face kernel (boundary.cu) refreshes the
-// ghosts of the new field after each step; under programmatic dependent launch
-// the next step starts while that kernel runs, and tiles whose halo touches a
-// face wait for it (griddepcontrol.wait), interior tiles do not.  When every
+// ghosts of the new field after each step.  When every
 // face is periodic and a row is a whole number of 32-byte sectors, the ghosts
 // are plain periodic images: the thread that writes a cell next to a face also
 // writes its image(s) on the far side (x images as whole 32-byte sectors of
-// the row pads, two threads a sector), so no face kernel runs, and the next
-// step waits for this one in every tile.
+// the row pads, two threads a sector), so no face kernel runs; where no face is
+// periodic the producer warp builds the ghosts of the planes it stages.  The
+// kernels of a call chain by programmatic dependent launch, each waiting for
+// the one before in every tile.
 //
 // Arithmetic.  From each plane every thread forms, for its cells,
 //   C  = phi at the cell,
@@ -302,6 +302,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
         " selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(ok)
         : "r"(smem_u32(bar)), "r"(parity), "r"(1000000u)
+        : "memory");
+    return ok != 0;
+}
+
+// One test of the phase that does not wait.
+__device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
     return ok != 0;
 }
@@ -707,7 +720,7 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                                           int by, int zc0, int zc1, S *__restrict__ stages,
                                           uint64_t *full, uint64_t *empty, int base, bool drain,
                                           int mode = 0, uint32_t sr_key = 0, uint64_t *ready = nullptr,
-                                          bool fwd = false)
+                                          bool fwd = false, bool wait = false)
 {
     static_assert(!SR || sizeof(T) == 4, "stochastic rounding is for FP32 compute");
     using Sh = TileShape<S, T, TX, TY, RPT_>;
@@ -723,98 +736,108 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
     const int tid = threadIdx.x;
     const int x0 = bx * W, y0 = by * TY;
     const int nplanes = zc1 - zc0 + 2;   // planes zc0-1 .. zc1
+    // the planes this tile stages hold ghosts that the producer warp has to build
+    const bool ghosts = fwd && (x0 == 0 || x0 + W >= g.nx || y0 == 0 || y0 + TY >= g.ny || zc0 == 0 || zc1 == g.nz);
 
     if (tid >= Sh::NCONS) {
         // ------------------------------------------------------- producer warp
-        // fwd (every face non-periodic): the whole warp builds the ghosts of the
-        // faces a staged plane touches (fix_xy, fix_z) and then releases it to
-        // the consumers on its "ready" barrier, NS - 2 planes behind the copies,
-        // so that as many copies stay in flight; otherwise one lane issues the
-        // copies and the consumers wait on "full".
+        // ghosts (a tile that touches a face of a grid whose faces are all
+        // non-periodic): the whole warp builds the ghosts of the faces a staged
+        // plane touches (fix_xy, fix_z) and then releases it to the consumers on
+        // its "ready" barrier; otherwise one lane issues the copies and the
+        // consumers wait on "full".
         const int plane_lane = tid - Sh::NCONS;
-        if (!fwd && plane_lane != 0) return true;
+        if (!ghosts && plane_lane != 0) return true;
         const bool lead = plane_lane == 0;
-        // The kernel may start while the previous launch still runs (programmatic
-        // dependent launch).  After a ghost-face refresh of src, a box that holds
-        // no ghost cell reads only interior cells, which the step before that
-        // wrote, so only boxes touching a face wait for the previous grid; after
-        // anything else (a step that wrote its own images, the first step of a
-        // call) every box waits.
-        if (lead && ((mode & kWaitAll) ||
-                     ((mode & kWaitFaces) &&
-                      (bx == 0 || x0 + W >= g.nx || by == 0 || y0 + TY >= g.ny || zc0 == 0 || zc1 == g.nz))))
-            asm volatile("griddepcontrol.wait;" ::: "memory");
+        // the kernel may start while the previous launch still runs (programmatic
+        // dependent launch): every box waits for it
+        if (lead && wait) asm volatile("griddepcontrol.wait;" ::: "memory");
         // kSkipCopy (a test of the bounded waits): the first CTA never fills the
         // stage of its plane 1, so its consumers' wait for that stage gives up
         const bool skip = (mode & kSkipCopy) && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
-        const bool zlo = fwd && zc0 == 0, zhi = fwd && zc1 == g.nz;
+        const bool zlo = ghosts && zc0 == 0, zhi = ghosts && zc1 == g.nz;
         auto stage = [&](int j) { return stages + ((base + j) % NS) * STAGE; };
-        // waits on the forwarding path suspend in hardware until the phase
-        // completes (no sleep back-off: the consumers wait behind them)
-        auto wait_full = [&](int j) {
-            return __all_sync(0xffffffffu, mbar_wait(&full[(base + j) % NS], ((base + j) / NS) & 1));
+        // the copy of plane i into its (free) stage
+        auto issue = [&](int i) {
+            const int s = (base + i) % NS;
+            // the ready barriers' phases go on with the ring, also where a tile of
+            // a batch does without them
+            if (fwd && !ghosts) mbar_arrive(&ready[s]);
+            if (skip && i == 1) return;
+            if (tmap) {
+                mbar_expect_tx(&full[s], (uint32_t)Sh::BOX_BYTES);
+                // one box: padded x from the 16-byte chunk left of the tile (x0 + off
+                // - VX, 16-byte aligned), padded rows y0.., padded plane zc0 + i;
+                // out-of-range parts are zero-filled, never used
+                tma_load_3d(stages + s * STAGE, tmap, x0 + g.off - VX, y0, zc0 + i, &full[s]);
+            } else {
+                // row by row (no tensor map): the box's rows that lie in the buffer
+                const long long row0 = (long long)(x0 + g.off - VX);
+                const int bytes_row = (int)min((long long)SW, (long long)g.pitch - row0) * (int)sizeof(S);
+                const int nrows = min(ROWS, g.ny + 2 - y0);
+                mbar_expect_tx(&full[s], (uint32_t)(bytes_row * nrows));
+                const S *plane = src + (long long)(zc0 + i) * g.plane + (long long)y0 * g.pitch + row0;
+                S *st = stages + s * STAGE;
+                for (int r = 0; r < nrows; ++r)
+                    bulk_g2s(st + r * SW, plane + (long long)r * g.pitch, (uint32_t)bytes_row, &full[s]);
+            }
         };
         auto release = [&](int j) {
             __syncwarp();
             if (lead) mbar_arrive(&ready[(base + j) % NS]);
         };
-        // plane j to the consumers: its x/y ghosts, or (a z ghost plane) all of it
-        // from the adjacent interior plane; plane 0 of a z- face follows plane 1
-        auto forward = [&](int j) -> bool {
-            if (zlo && j == 0) return true;
-            if (!wait_full(j)) return false;
-            if (zhi && j == nplanes - 1) fix_z<S, T, SW, ROWS>(stage(j), stage(j - 1), g, C.aface, 5, plane_lane);
-            else fix_xy<S, T, VX, SW, ROWS>(stage(j), g, C.aface, x0, y0, W, TY, plane_lane);
-            release(j);
-            if (zlo && j == 1) {
-                if (!wait_full(0)) return false;
-                fix_z<S, T, SW, ROWS>(stage(0), stage(1), g, C.aface, 4, plane_lane);
-                release(0);
-            }
-            return true;
-        };
-        // lag NS - 2: plane 0 of a z- face, forwarded with plane 1, is released
-        // before the copy of plane NS has to wait for its stage
-        const int lag = fwd ? NS - 2 : 0;
         int issued = 0;
         bool ok = true;
-        for (int i = 0; i < nplanes + lag; ++i) {
-            if (i < nplanes) {
-                if (lead) {
-                    const int I = base + i, s = I % NS;
-                    if (I >= NS && !(fwd ? mbar_wait(&empty[s], ((I / NS) - 1) & 1)
-                                         : mbar_wait_sleep(&empty[s], ((I / NS) - 1) & 1))) {
-                        ok = false;
-                    } else if (!(skip && i == 1)) {
-                        if (tmap) {
-                            mbar_expect_tx(&full[s], (uint32_t)Sh::BOX_BYTES);
-                            // one box: padded x from the 16-byte chunk left of the tile (x0 + off
-                            // - VX, 16-byte aligned), padded rows y0.., padded plane zc0 + i;
-                            // out-of-range parts are zero-filled, never used
-                            tma_load_3d(stages + s * STAGE, tmap, x0 + g.off - VX, y0, zc0 + i, &full[s]);
-                        } else {
-                            // row by row (no tensor map): the box's rows that lie in the buffer
-                            const long long row0 = (long long)(x0 + g.off - VX);
-                            const int bytes_row = (int)min((long long)SW, (long long)g.pitch - row0) * (int)sizeof(S);
-                            const int nrows = min(ROWS, g.ny + 2 - y0);
-                            mbar_expect_tx(&full[s], (uint32_t)(bytes_row * nrows));
-                            const S *plane = src + (long long)(zc0 + i) * g.plane + (long long)y0 * g.pitch + row0;
-                            S *st = stages + s * STAGE;
-                            for (int r = 0; r < nrows; ++r)
-                                bulk_g2s(st + r * SW, plane + (long long)r * g.pitch, (uint32_t)bytes_row, &full[s]);
-                        }
-                    }
-                    if (ok) ++issued;
+        if (!ghosts) {
+            for (; issued < nplanes; ++issued) {
+                const int I = base + issued;
+                if (I >= NS && !mbar_wait_sleep(&empty[I % NS], ((I / NS) - 1) & 1)) {
+                    ok = false;
+                    break;
                 }
-                if (fwd) ok = __shfl_sync(0xffffffffu, ok, 0) != 0;
-                if (!ok) break;
+                issue(issued);
             }
-            if (fwd && i >= lag && !forward(i - lag)) {
-                ok = false;
-                break;
+        } else {
+            // Copies and releases go on independently, whichever can: a copy when its
+            // stage is free, a plane's release when it has landed, in order (plane 0
+            // of a z- face, which is built from plane 1, after that one).  A fixed
+            // lag of the releases behind the copies left the consumers one plane of
+            // slack.
+            int done = 0;
+            long long idle_since = 0;
+            while (done < nplanes) {
+                bool moved = false;
+                if (issued < nplanes) {
+                    const int I = base + issued;
+                    if (I < NS || __all_sync(0xffffffffu, mbar_test(&empty[I % NS], ((I / NS) - 1) & 1))) {
+                        if (lead) issue(issued);
+                        ++issued;
+                        moved = true;
+                    }
+                }
+                const int j = zlo && done < 2 ? 1 - done : done;
+                if (j < issued && __all_sync(0xffffffffu, mbar_test(&full[(base + j) % NS], ((base + j) / NS) & 1))) {
+                    if (zlo && j == 0) fix_z<S, T, SW, ROWS>(stage(0), stage(1), g, C.aface, 4, plane_lane);
+                    else if (zhi && j == nplanes - 1)
+                        fix_z<S, T, SW, ROWS>(stage(j), stage(j - 1), g, C.aface, 5, plane_lane);
+                    else fix_xy<S, T, VX, SW, ROWS>(stage(j), g, C.aface, x0, y0, W, TY, plane_lane);
+                    release(j);
+                    ++done;
+                    moved = true;
+                }
+                if (moved) {
+                    idle_since = 0;
+                } else {
+                    const long long now = clock64();
+                    if (idle_since == 0) idle_since = now;
+                    if (__any_sync(0xffffffffu, now - idle_since > kWaitCycles)) {
+                        ok = false;
+                        break;
+                    }
+                    __nanosleep(40);
+                }
             }
         }
-        if (fwd) issued = __shfl_sync(0xffffffffu, issued, 0);
         if (!lead) return ok;
         if (!ok) atomicOr(err, 1);
         // never leave with copies in flight: wait for each stage's copy (a stage
@@ -854,7 +877,7 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                     PlaneQ<T, NP> (&p)[RPT]) -> bool {
         const int I = base + i, s = I % NS;
         // warp-uniform: every lane waits (acquire), the warp goes on only if all saw it
-        if (!__all_sync(0xffffffffu, mbar_wait(fwd ? &ready[s] : &full[s], (I / NS) & 1))) {
+        if (!__all_sync(0xffffffffu, mbar_wait(ghosts ? &ready[s] : &full[s], (I / NS) & 1))) {
             if (lane == 0) atomicOr(err, 4);
             ok = false;
             return false;
@@ -1139,10 +1162,7 @@ __global__ void __launch_bounds__(TileShape<S, T, TX, TY, RPT_>::NTHREADS,
                      const __grid_constant__ CUtensorMap tmap, int use_tmap, int mode)
 {
     using Sh = TileShape<S, T, TX, TY, RPT_>;
-    // a step that writes its own ghost images, or whose grid has no periodic face
-    // (no face kernel follows), lets the next step launch at once: every box of
-    // that step waits for this grid (kWaitAll) before it reads
-    if (IMG || (mode & kEarly)) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (mode & kEarly) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ __align__(128) S stages[Sh::NS * Sh::STAGE];
     __shared__ __align__(8) uint64_t full[Sh::NS], empty[Sh::NS], ready[Sh::NS];
     if (threadIdx.x == 0) {
@@ -1165,7 +1185,8 @@ __global__ void __launch_bounds__(TileShape<S, T, TX, TY, RPT_>::NTHREADS,
     }
     step_tile<S, T, STENCIL, KIND, TX, TY, RPT_, IMG, SR>(C, PC, src, dst, err, use_tmap ? &tmap : nullptr,
                                                      blockIdx.x, blockIdx.y, zc0, zc1, stages, full, empty, 0,
-                                                     true, mode, C.sr_key, ready, fwd);
+                                                     true, mode, C.sr_key, ready, fwd, true);
+    if (!(mode & kEarly)) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // ------------------------------------------------------------------- batches
@@ -1208,7 +1229,8 @@ __global__ void __launch_bounds__(TileShape<S, T, TX, TY>::NTHREADS, kBatchCtasP
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;" ::: "memory");
+    if (list.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     int base = 0;
     const int end = list.start[blockIdx.x + 1];
     for (int w = list.start[blockIdx.x]; w < end; ++w) {
@@ -1226,6 +1248,7 @@ __global__ void __launch_bounds__(TileShape<S, T, TX, TY>::NTHREADS, kBatchCtasP
             return;
         base += it.zc1 - it.zc0 + 2;
     }
+    if (!list.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Work-list entries of one grid for the tile shape (TX, TY) of the (S, T)
@@ -1315,7 +1338,7 @@ cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, 
     lc.stream = st;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    const int mode = cfg.mode;
+    int mode = cfg.mode;
     // z-chunk: the caller's, else the launch-shape model's for this kernel (a
     // grid dimension stays below 65536 chunks)
     auto go = [&](auto kern, int threads) {
@@ -1326,6 +1349,7 @@ cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, 
         if (zchunk < (c.g.nz + 65534) / 65535) zchunk = (c.g.nz + 65534) / 65535;
         if (cfg.zchunk_used) *cfg.zchunk_used = zchunk;
         lc.gridDim = dim3(gxn, gyn, (c.g.nz + zchunk - 1) / zchunk);
+        if ((long long)gxn * gyn * lc.gridDim.z >= 4LL * sms * MinBlocks<S>::value) mode |= kEarly;
         lc.blockDim = dim3(threads);
         return cudaLaunchKernelEx(&lc, kern, c, pc, src, dst, err, zchunk, map, use, mode);
     };
