@@ -481,20 +481,14 @@ template <class S> struct MantBits;
 template <> struct MantBits<float> { static constexpr int v = 23; };
 template <> struct MantBits<__nv_bfloat16> { static constexpr int v = 7; };
 
-// spacing of S above a >= 0 (from a's exponent; 0 for |a| < 2^(bits - 126))
-__device__ __forceinline__ float spacing_above(float a, int bits)
-{
-    const int e = (int)(__float_as_uint(a) & 0x7f800000u) - (bits << 23);
-    return __int_as_float(e > 0 ? e : 0);
-}
-
-// the largest BF16 value not above v (v an FP32 value)
+// the largest BF16 value not above v (an FP32 value): truncation, away from zero
+// where v is negative
 __device__ __forceinline__ float bf16_round_down(float v)
 {
-    uint32_t b = __float_as_uint(v);
-    if ((b & 0x80000000u) && (b & 0xffffu)) b = (b & 0xffff0000u) + 0x10000u;   // away from zero
-    else b &= 0xffff0000u;
-    return __uint_as_float(b);
+    const uint32_t b = __float_as_uint(v);
+    uint32_t low;   // 0xffff where the sign bit is set (the top byte's sign, replicated)
+    asm("prmt.b32 %0, %1, 0, 0x44bb;" : "=r"(low) : "r"(b));
+    return __uint_as_float((b + low) & 0xffff0000u);
 }
 
 template <class S>
@@ -503,11 +497,15 @@ __device__ __forceinline__ float2 sr_update(float2 ph, float2 inc, uint32_t h)
     constexpr int mb = MantBits<S>::v;
     float2 a = __fadd2_rd(ph, inc);
     if constexpr (mb == 7) { a.x = bf16_round_down(a.x); a.y = bf16_round_down(a.y); }
-    const float2 g = make_float2(spacing_above(fabsf(a.x), mb), spacing_above(fabsf(a.y), mb));
-    const float2 u = __fadd2_rn(make_float2(__uint_as_float(0x3f800000u | ((h << 7) & 0x007fff80u)),
-                                            __uint_as_float(0x3f800000u | ((h >> 9) & 0x007fff80u))),
-                                make_float2(-1.0f, -1.0f));
-    float2 x = __fadd2_rd(ph, __ffma2_rn(u, g, inc));
+    // the power of two of a; times u 2^-mb, u g of above (u 2^-mb is exact: its 16
+    // bits in the mantissa of (1 + u) 2^-mb)
+    const float2 p = make_float2(__uint_as_float(__float_as_uint(a.x) & 0x7f800000u),
+                                 __uint_as_float(__float_as_uint(a.y) & 0x7f800000u));
+    constexpr uint32_t one = (uint32_t)(127 - mb) << 23;   // 2^-mb
+    const float2 u = __fadd2_rn(make_float2(__uint_as_float(one | ((h << 7) & 0x007fff80u)),
+                                            __uint_as_float(one | ((h >> 9) & 0x007fff80u))),
+                                make_float2(-__uint_as_float(one), -__uint_as_float(one)));
+    float2 x = __fadd2_rd(ph, __ffma2_rn(u, p, inc));
     if constexpr (mb == 7) { x.x = bf16_round_down(x.x); x.y = bf16_round_down(x.y); }
     return x;
 }
