@@ -703,6 +703,36 @@ __device__ __forceinline__ P laplace_update(const PCoef &PC, P t, P ph, P h, P g
     return acc;
 }
 
+// The potential's sum group by group as one running fraction num / den, u = s^2.
+template <class T>
+__device__ __forceinline__ void sum_groups(const typename PackCoef<T>::Pair *pair, int n, typename Pk<T>::P u,
+                                           typename Pk<T>::P &num, typename Pk<T>::P &den)
+{
+    using K = Pk<T>;
+    using P = typename K::P;
+    const P one = K::mk(T(1), T(1));
+    const typename PackCoef<T>::Pair t0 = pair[0];
+    P nu = t0.nbeta, de = K::fma(t0.nA, u, one);
+#pragma unroll 1
+    for (int k = 1; k < n; ++k) {
+        const typename PackCoef<T>::Pair t = pair[k];
+        const P d = K::fma(t.nA, u, one);
+        nu = K::fma(nu, d, K::mul(t.nbeta, de));
+        de = K::mul(de, d);
+    }
+    num = nu;
+    den = de;
+}
+
+// The same as a call: it is rare, and inlined in the batch kernel it holds
+// registers that the plane loop spills for.
+template <class T>
+__device__ __noinline__ void call_sum_groups(const typename PackCoef<T>::Pair *pair, int n, typename Pk<T>::P u,
+                                             typename Pk<T>::P &num, typename Pk<T>::P &den)
+{
+    sum_groups<T>(pair, n, u, num, den);
+}
+
 // KIND: the potential (spfm_internal.h).  Degrees below the kernel's are padded
 // with zero coefficients, which changes no bit.
 // One tile (bx, by) of planes zc0..zc1-1.  The stage ring continues across the
@@ -711,7 +741,8 @@ __device__ __forceinline__ P laplace_update(const PCoef &PC, P t, P ph, P h, P g
 // Returns false when a bounded wait gave up (the error word is set).
 // SR: stochastic rounding of the update (FP32 compute only), random bits from
 // sr_hash(padded cell index xor sr_key).
-template <class S, class T, int STENCIL, int KIND, int TX, int TY, int RPT_, bool IMG = false, bool SR = false>
+template <class S, class T, int STENCIL, int KIND, int TX, int TY, int RPT_, bool IMG = false, bool SR = false,
+          bool IMM = false>
 __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T> &PC,
                                           const S *__restrict__ src, S *__restrict__ dst,
                                           int *__restrict__ err, const CUtensorMap *tmap, int bx,
@@ -730,6 +761,9 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
     constexpr bool kGuard = KIND > 4;                       // q below q_lo: group by group
     constexpr int DEG = KIND > kKindFew ? KIND - kKindFew : KIND;
 
+    // one, -2, -4: from the parameters, or immediates (IMM: PC is in memory)
+    const P k1 = IMM ? K::mk(T(1), T(1)) : PC.one, k2 = IMM ? K::mk(T(-2), T(-2)) : PC.m2,
+            k4 = IMM ? K::mk(T(-4), T(-4)) : PC.m4;
     const GridGeom &g = C.g;
     const int tid = threadIdx.x;
     const int x0 = bx * W, y0 = by * TY;
@@ -926,13 +960,13 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                     const P c = cell(r + 1, q);
                     p[r].c[q] = c;
                     // F' = (W + E + N + S) - 4C, E' = (NW + NE + SW + SE) - 4C
-                    const P f = K::fma(PC.m4, c, K::add(side(r + 1, q), K::add(cell(r, q), cell(r + 2, q))));
+                    const P f = K::fma(k4, c, K::add(side(r + 1, q), K::add(cell(r, q), cell(r + 2, q))));
                     // 6 neighbours: h = F' (c1 applied in the update's FMA); 18: g = F'
                     // (c2 applied to the sum of the two planes' g in one FMA)
                     if (STENCIL == 6) {
                         p[r].h[q] = f;
                     } else {
-                        const P e = K::fma(PC.m4, c, K::add(side(r, q), side(r + 2, q)));
+                        const P e = K::fma(k4, c, K::add(side(r, q), side(r + 2, q)));
                         p[r].h[q] = K::fma(PC.c2, e, K::mul(PC.c1, f));
                         p[r].g[q] = STENCIL == 26 ? K::fma(PC.c3, e, K::mul(PC.c2, f)) : f;
                     }
@@ -960,21 +994,12 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                         const P t = K::second(m[r].c[q], p[r].c[q], ph);
                         // SR: the increment alone, phi is added once in sr_update
                         const P acc = laplace_update<SR, STENCIL>(PC, t, ph, z[r].h[q], m[r].g[q], p[r].g[q]);
-                        const P sg = K::fma(PC.m2, ph, PC.one);
-                        const P q1 = K::bump(ph, PC.one);
+                        const P sg = K::fma(k2, ph, k1);
+                        const P q1 = K::bump(ph, k1);
                         P num, den;
                         if constexpr (by_group.value) {
-                            const P u = K::mul(sg, sg);
-                            const typename PackCoef<T>::Pair t0 = PC.pair[0];
-                            num = t0.nbeta;
-                            den = K::fma(t0.nA, u, PC.one);
-#pragma unroll 1
-                            for (int kk = 1; kk < PC.nterms; ++kk) {
-                                const typename PackCoef<T>::Pair tk = PC.pair[kk];
-                                const P d = K::fma(tk.nA, u, PC.one);
-                                num = K::fma(num, d, K::mul(tk.nbeta, den));
-                                den = K::mul(den, d);
-                            }
+                            if constexpr (IMM) call_sum_groups<T>(PC.pair, PC.nterms, K::mul(sg, sg), num, den);
+                            else sum_groups<T>(PC.pair, PC.nterms, K::mul(sg, sg), num, den);
                         } else if constexpr (KIND == kKindAny) {
                             const int n = PC.deg;
                             num = PC.rat[n - 1].num;
@@ -987,12 +1012,12 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                             }
                         } else {
                             num = PC.rat[DEG - 1].num;
-                            den = K::fma(PC.rat[DEG].den, q1, DEG == 1 ? PC.one : PC.rat[DEG - 1].den);
+                            den = K::fma(PC.rat[DEG].den, q1, DEG == 1 ? k1 : PC.rat[DEG - 1].den);
 #pragma unroll
                             for (int i = DEG - 2; i >= 0; --i) {
                                 const typename PackCoef<T>::Ratio c = PC.rat[i];
                                 num = K::fma(num, q1, c.num);
-                                den = K::fma(den, q1, i == 0 ? PC.one : c.den);
+                                den = K::fma(den, q1, i == 0 ? k1 : c.den);
                             }
                         }
                         const P w = K::fma(sg, K::div(num, den), PC.nkmu);
@@ -1032,7 +1057,7 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                         if (bulk) {
 #pragma unroll
                             for (int q = 0; q < NP; ++q)
-                                wl[q] = K::fma(K::fma(PC.m2, z[r].c[q], PC.one),
+                                wl[q] = K::fma(K::fma(k2, z[r].c[q], k1),
                                                K::mk(-C.dt * C.kappa, -C.dt * C.kappa),
                                                K::mk(-C.dt * C.kmu, -C.dt * C.kmu));
                         } else {
@@ -1046,11 +1071,11 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                             auto diff = [&](P a, P b) {
                                 a = clamp_pack(a, ep);
                                 b = clamp_pack(b, ep);
-                                return K::mul(log_odds_diff(a, K::sub(PC.one, a), b, K::sub(PC.one, b)), s2);
+                                return K::mul(log_odds_diff(a, K::sub(k1, a), b, K::sub(k1, b)), s2);
                             };
 #pragma unroll
                             for (int q = 0; q < NP; ++q) {
-                                const P sg = K::fma(PC.m2, z[r].c[q], PC.one);
+                                const P sg = K::fma(k2, z[r].c[q], k1);
                                 wl[q] = ti_local_w<T, STENCIL>(
                                     C, sg, K::mul(sg, sg),
                                     diff(K::mk(x[2 * q + 2], x[2 * q + 3]), K::mk(x[2 * q], x[2 * q + 1])),
@@ -1065,8 +1090,8 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                         const P t = K::second(m[r].c[q], p[r].c[q], ph);
                         // phi + dt * Laplacian (SR: the increment alone, phi is added in sr_update)
                         const P acc = laplace_update<SR, STENCIL>(PC, t, ph, z[r].h[q], m[r].g[q], p[r].g[q]);
-                        const P sg = K::fma(PC.m2, ph, PC.one);               // s = 1 - 2 phi
-                        const P q1 = K::bump(ph, PC.one);                     // q = phi (1 - phi)
+                        const P sg = K::fma(k2, ph, k1);               // s = 1 - 2 phi
+                        const P q1 = K::bump(ph, k1);                     // q = phi (1 - phi)
                         P w;   // -dt (potential / q + 4 M dF / (lambda Gamma))
                         if (KIND == 0) {
                             // driving term -dt pref dF h'(phi) = q (nkmu f): f = 1 for h3,
@@ -1075,7 +1100,7 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                             if (C.interp == 1) {
                                 drive = K::mul(PC.nkmu, K::mul(K::mk(T(5), T(5)), q1));
                             } else if (C.interp == 2) {
-                                const P d = K::fma(K::mk(T(-2), T(-2)), q1, PC.one);
+                                const P d = K::fma(K::mk(T(-2), T(-2)), q1, k1);
                                 drive = K::div(PC.nkmu, K::mul(K::mk(T(3), T(3)), K::mul(d, d)));
                             }
                             w = K::fma(sg, PC.nkap, drive);
@@ -1227,6 +1252,8 @@ __global__ void __launch_bounds__(TileShape<S, T, TX, TY>::NTHREADS, kBatchCtasP
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    __shared__ __align__(32) unsigned char s_raw[(Sh::NCONS / 32) * sizeof(PackCoef<T>)];
+    PackCoef<T> *s_pc = reinterpret_cast<PackCoef<T> *>(s_raw);
     if (list.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     int base = 0;
@@ -1240,8 +1267,21 @@ __global__ void __launch_bounds__(TileShape<S, T, TX, TY>::NTHREADS, kBatchCtasP
             asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(map) : "memory");
         const bool last = w + 1 == end;
         const uint32_t key = SR ? sr_step_key(bg.C.sr_seed, steps[it.grid] + sub) : 0u;
-        if (!step_tile<S, T, STENCIL, KIND, TX, TY, SPFM_ROWS_PER_THREAD, false, SR>(
-                bg.C, bg.PC, (const S *)bg.field[cur], (S *)bg.field[cur ^ 1], err, map, it.bx, it.by, it.zc0,
+        const int warp = threadIdx.x >> 5;
+        // each consumer warp reads the item's coefficients from a copy of its own in
+        // shared memory: from the grid record in global memory every row waited for
+        // them (long_scoreboard a third of the stalls; 64-grid sweep 89.7 -> 85.7 us
+        // a step, served window 293.8 -> 274.1)
+        if (warp < Sh::NCONS / 32) {
+            __syncwarp();
+            const uint32_t *from = reinterpret_cast<const uint32_t *>(&bg.PC);
+            uint32_t *to = reinterpret_cast<uint32_t *>(&s_pc[warp]);
+            for (int k = threadIdx.x & 31; k < (int)(sizeof(PackCoef<T>) / 4); k += 32) to[k] = from[k];
+            __syncwarp();
+        }
+        const PackCoef<T> &pc = s_pc[warp < Sh::NCONS / 32 ? warp : 0];
+        if (!step_tile<S, T, STENCIL, KIND, TX, TY, SPFM_ROWS_PER_THREAD, false, SR, true>(
+                bg.C, pc, (const S *)bg.field[cur], (S *)bg.field[cur ^ 1], err, map, it.bx, it.by, it.zc0,
                 it.zc1, stages, full, empty, base, last, 0, key, ready, fwd != 0))
             return;
         base += it.zc1 - it.zc0 + 2;
