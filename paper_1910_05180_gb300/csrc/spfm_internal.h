@@ -216,7 +216,7 @@ constexpr int kImages = 4, kSkipCopy = 8, kEarly = 16;
 
 // TMA tensor maps of a grid's two field buffers, encoded on first use (tma.cu).
 struct TmaCache {
-    CUtensorMap map[4];   // [buffer] for the single-grid box, [2 + buffer] for the square batch box
+    CUtensorMap map[4];   // [buffer] for the single-grid box, [2 + buffer] for the square box
     const void *base[4];
     int state[4];   // 0 not encoded, 1 encoded, -1 encoding unavailable (row copies)
 };

@@ -8,8 +8,7 @@ namespace spfm {
 cudaError_t launch_step_f32_img_sr(const StepCoef<float> &c, const float *src, float *dst, int *err,
                                    LaunchCfg cfg, TmaCache *tma, int which, cudaStream_t st)
 {
-    using Sh = TileShape<float, float, SPFM_F32_TX, SPFM_F32_TY>;
-    const CUtensorMap *map = cached_map(tma, which, c.g, SPFM_F32, src, Sh::SW, Sh::ROWS);
-    return launch_step_t<float, float, SPFM_F32_TX, SPFM_F32_TY, true, true>(c, src, dst, err, cfg, map, st);
+    const CUtensorMap *map = f32_step_map(tma, which, c, cfg.scheme, src);
+    return launch_step_t<float, float, SPFM_F32_TX, SPFM_F32_TY, true, true, kSqTX, kSqTY>(c, src, dst, err, cfg, map, st);
 }
 }  // namespace spfm

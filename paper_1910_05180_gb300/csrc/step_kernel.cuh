@@ -1344,17 +1344,33 @@ cudaError_t launch_batch_t(const void *grids, BatchList list, int parity, int *e
 }
 
 // IMG: the kernels that write the periodic ghost images (cfg.mode has kImages)
-template <class S, class T, int TX, int TY, bool IMG, bool SR = false>
+// TI_n on the square tile LTX, LTY (tmap is then that tile's map)?  A warp of it
+// covers 32 x 4 cells instead of 64 x 2, so fewer warps touch the interface
+// band, whose cells cost several times those of the bulk; where the band fills
+// much of the grid that gains nothing and the tile's wider x halo costs.  The
+// line lies at an extent of 32 lambda, about 4.5 band widths (FP32 27-point, us a
+// step, wide -> square: lambda = 3: 320^3 118.6 -> 112.1, 96^3 14.1 -> 12.2;
+// lambda = 6: 256^3 88.0 -> 79.4, 192^3 55.8 -> 57.3, 128^3 23.3 -> 24.7).
+template <class T>
+inline bool local_square(const StepCoef<T> &c, int scheme)
+{
+    const int n = min(c.g.nx, min(c.g.ny, c.g.nz));
+    return scheme == SPFM_TI_LOCAL && n * c.two_dx_over_lam >= T(64);
+}
+
+template <class S, class T, int TX, int TY, bool IMG, bool SR = false, int LTX = TX, int LTY = TY>
 cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, LaunchCfg cfg,
                           const CUtensorMap *tmap, cudaStream_t st)
 {
-    using Sh = TileShape<S, T, TX, TY>;
-    const int gxn = (c.g.nx + Sh::W - 1) / Sh::W, gyn = (c.g.ny + TY - 1) / TY;
+    using Lo = TileShape<S, T, LTX, LTY, 1>;
+    const int kind = grid_kind(cfg.scheme, c.deg, isinf(c.q_lo));
+    const bool square = LTX != TX && local_square(c, cfg.scheme);
+    const int tw = square ? Lo::W : TileShape<S, T, TX, TY>::W, th = square ? LTY : TY;
+    const int gxn = (c.g.nx + tw - 1) / tw, gyn = (c.g.ny + th - 1) / th;
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int target = 6 * MinBlocks<S>::value * sms;
-    const int kind = grid_kind(cfg.scheme, c.deg, isinf(c.q_lo));
     const PackCoef<T> pc = make_pack_coef<T>(c);
     CUtensorMap map;
     if (tmap) map = *tmap;
@@ -1403,6 +1419,7 @@ cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, 
         else if (kind == kKindFew + 4) SPFM_LAUNCH(ST, kKindFew + 4); \
         else if (kind == kKindFew + 6) SPFM_LAUNCH(ST, kKindFew + 6); \
         else if (kind == kKindAny) SPFM_LAUNCH(ST, kKindAny); \
+        else if (square) le = go(spfm_step_kernel<S, T, ST, kKindLocal, LTX, LTY, 1, IMG, SR>, Lo::NTHREADS); \
         else le = go(spfm_step_kernel<S, T, ST, kKindLocal, TX, TY, 1, IMG, SR>, NT1); \
     } while (0)
     if (cfg.stencil == 6) SPFM_BY_KIND(6);
