@@ -253,15 +253,15 @@ __device__ __forceinline__ long long fix48(float y)
 }
 
 // Volume of one lane.  FP32 values: each row as an unevaluated pair s + c
-// (TwoSum), then the pair in 2^-48 fixed point (exact to the dropped bits,
-// below 4e-15 per row), carried into FP64 every 64 rows, before the fixed
+// (TwoSum) over four rows, then the pair in 2^-48 fixed point (exact to the
+// dropped bits, below 4e-15 per four rows), carried into FP64 before the fixed
 // point could overflow.
 template <class R> struct VolSum;
 template <> struct VolSum<float> {
     float2 s = {0.0f, 0.0f}, c = {0.0f, 0.0f};   // two chains
     long long fix = 0;
     double sum = 0.0;
-    int rows = 0;
+    int rows = 0, flushes = 0;
     static __device__ __forceinline__ float2 sub(float2 a, float2 b)
     {
         return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
@@ -280,20 +280,29 @@ template <> struct VolSum<float> {
         s = make_float2(r.x, r.y);
         c = make_float2(r.z, r.w);
     }
-    __device__ __forceinline__ void end_row()
+    // the chains into fixed point (every fourth row: a row of 512 cells is 16 a lane)
+    __device__ __forceinline__ void flush()
     {
         const DF t = df_two_sum(s.x, s.y);
         const float lo = (c.x + c.y) + t.lo;
         if (fabsf(t.hi) < 256.0f) fix += fix48(t.hi) + fix48(lo);
         else sum += (double)t.hi + (double)lo;
         set_row(make_float4(0.0f, 0.0f, 0.0f, 0.0f));
-        if (++rows == 64) {
+        if (++flushes == 32) {
             sum += (double)fix * 0x1p-48;
             fix = 0;
-            rows = 0;
+            flushes = 0;
         }
     }
-    __device__ __forceinline__ double total() const { return sum + (double)fix * 0x1p-48; }
+    __device__ __forceinline__ void end_row()
+    {
+        if ((++rows & 3) == 0) flush();
+    }
+    __device__ __forceinline__ double total()
+    {
+        flush();
+        return sum + (double)fix * 0x1p-48;
+    }
 };
 template <> struct VolSum<double> {
     double sum = 0.0;
@@ -463,13 +472,14 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
             }
             // extrema and volume of the lane's whole pieces (a piece that a row's
             // end cuts goes cell by cell), and whether any cell may lie in the band
-            bool near = false;
+            unsigned parts = 0u;   // bit p: one of the lane's cells 4 p .. 4 p + 3 may lie in the band
             R lo = R(INFINITY), hi = R(-INFINITY);
             if constexpr (sizeof(R) == 4) {
-                float far = 1.0f;   // the least |phi - 1/2|
 #pragma unroll
                 for (int t = 0; t < V; ++t) {
+                    constexpr unsigned kPiece = (1u << (E / 4)) - 1u;   // its parts
                     const int vi = v0 + 32 * t + lane;
+                    float far = 1.0f;   // the least |phi - 1/2|; band cells have less than 1/2 - 1e-6
                     if (vi < nwhole) {
 #pragma unroll
                         for (int e = 0; e < E; e += 2) {
@@ -480,19 +490,23 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
                             const float2 d = __fadd2_rn(x, make_float2(-0.5f, -0.5f));
                             far = fminf(fminf(far, fabsf(d.x)), fabsf(d.y));
                         }
-                    } else if (vi < nvec) {
-#pragma unroll
-                        for (int e = 0; e < E; ++e)
-                            if (vi * E + e < a.g.nx) {
-                                const float x = Row16<S>::get(w[t], e);
-                                near = near || in_band(x);
-                                vol.add(x);
-                                lo = fminf(lo, x);
-                                hi = fmaxf(hi, x);
-                            }
+                    }
+                    if (far < 0.5f - 0.5e-6f) parts |= kPiece << (t * E / 4);
+                }
+                // the piece that the row's end cuts, where the sweep holds it (a warp's
+                // branch, so that other sweeps do not pass through this code)
+                if (nwhole < nvec && nwhole >= v0 && nwhole < v0 + 32 * V) {
+                    const int t = (nwhole - v0) / 32;
+                    if (v0 + 32 * t + lane == nwhole) {
+                        for (int i = nwhole * E; i < a.g.nx; ++i) {
+                            const float x = scr<S>(reinterpret_cast<const S *>(src), i);
+                            if (in_band(x)) parts |= 1u << ((t * E + i - nwhole * E) / 4);
+                            vol.add(x);
+                            lo = fminf(lo, x);
+                            hi = fmaxf(hi, x);
+                        }
                     }
                 }
-                near = near || far < 0.5f - 0.5e-6f;   // band cells have |phi - 1/2| < 1/2 - 1e-6
                 if (!vol.finite()) {   // the sweep again, without the cells that are not
                     vol.set_row(before);
                     lo = R(INFINITY);
@@ -530,36 +544,15 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
                             const long long k = order_key(x);
                             klo = k < klo ? k : klo;
                             khi = k > khi ? k : khi;
-                            near = near || h - 0x3eb0c6f7u <= 0x3feffffeu - 0x3eb0c6f7u;
+                            if (h - 0x3eb0c6f7u <= 0x3feffffeu - 0x3eb0c6f7u) parts |= 1u << ((t * E + e) / 4);
                         }
             }
             if constexpr (sizeof(R) == 4) {
                 mn = fewest(mn, lo);
                 mx = most(mx, hi);
             }
-            if (!__any_sync(0xffffffffu, near)) continue;
-            unsigned bm = 0u;   // band cells of this lane among its E * V
-#pragma unroll
-            for (int t = 0; t < V; ++t)
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    const R x = Row16<S>::get(w[t], e);
-                    if (in_band(x) && (v0 + 32 * t + lane) * E + e < a.g.nx) bm |= 1u << (t * E + e);
-                }
-            if (__any_sync(0xffffffffu, bm != 0u)) {
-                if (!row_known) {
-                    // the row's shares of p.n and |p - ctr|^2, in double-float (FP64
-                    // is the slow pipe of this GPU)
-                    slot = band_rows++ & (kRowSlots - 1);
-                    if (lane == 0) {
-                        const DF fj = df_of_int(j), fk = df_of_int(k);
-                        const DF ry = df_add(df_mul(bconst.dx, fj), bconst.neg_c1);
-                        const DF rz = df_add(df_mul(bconst.dx, fk), bconst.neg_c2);
-                        row_tab[warp][slot][0] = df_add(df_mul(bconst.dxn1, fj), df_mul(bconst.dxn2, fk));
-                        row_tab[warp][slot][1] = df_add(df_mul(ry, ry), df_mul(rz, rz));
-                    }
-                    row_known = true;
-                }
+            parts = __reduce_or_sync(0xffffffffu, parts);   // of any lane
+            if (parts != 0u) {
                 // Queue the sweep's band cells in four parts of 4 cells a lane (a warp
                 // prefix sum places each lane's), evaluating full warps after each.
                 // The parts stay a loop, the sweep's words moving down by one part a
@@ -575,9 +568,30 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
                     u[4 * t + 3] = w[t].w;
                 }
 #pragma unroll 1
-                for (int part = 0; part < 4; ++part) {
-                    const unsigned m = bm & 0xfu;
+                for (int part = 0; parts != 0u; ++part, parts >>= 1) {
+                    unsigned m = 0u;   // the lane's band cells of the part
+                    if (parts & 1u) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int b = 4 * part + k;   // cell of the lane's E * V
+                            if (in_band(word_cell<S>(u, k)) && (v0 + 32 * (b / E) + lane) * E + b % E < a.g.nx)
+                                m |= 1u << k;
+                        }
+                    }
                     if (__any_sync(0xffffffffu, m != 0u)) {
+                        if (!row_known) {
+                            // the row's shares of p.n and |p - ctr|^2, in double-float (FP64
+                            // is the slow pipe of this GPU)
+                            slot = band_rows++ & (kRowSlots - 1);
+                            if (lane == 0) {
+                                const DF fj = df_of_int(j), fk = df_of_int(k);
+                                const DF ry = df_add(df_mul(bconst.dx, fj), bconst.neg_c1);
+                                const DF rz = df_add(df_mul(bconst.dx, fk), bconst.neg_c2);
+                                row_tab[warp][slot][0] = df_add(df_mul(bconst.dxn1, fj), df_mul(bconst.dxn2, fk));
+                                row_tab[warp][slot][1] = df_add(df_mul(ry, ry), df_mul(rz, rz));
+                            }
+                            row_known = true;
+                        }
                         const int c = __popc(m);
                         int incl = c;
 #pragma unroll
@@ -590,7 +604,7 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
                         for (int k = 0; k < 4; ++k) {
                             if (m & (1u << k)) {
                                 const int r = pos & (kRing - 1);
-                                const int b = 4 * part + k;   // cell of the lane's E * V
+                                const int b = 4 * part + k;
                                 ring_phi[warp][r] = word_cell<S>(u, k);
                                 ring_i[warp][r] = (v0 + 32 * (b / E) + lane) * E + b % E;
                                 ring_slot[warp][r] = (unsigned char)slot;
@@ -602,7 +616,6 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
                         for (; tail - head >= 32; head += 32) eval_at(head + lane);
                         __syncwarp();   // reads of evaluated cells before the next part's writes
                     }
-                    bm >>= 4;
 #pragma unroll
                     for (int k = 0; k + kW < 4 * V; ++k) u[k] = u[k + kW];
                 }
