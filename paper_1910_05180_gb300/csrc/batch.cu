@@ -161,10 +161,12 @@ struct Deal {
     std::vector<BatchItem> items;   // in CTA order, shape 0 first
     std::vector<int> starts;        // kMaxCtas + 1 entries a shape
     int ctas[2] = {0, 0}, nitems0 = 0;
+    size_t count = 0;               // items
     long long span = 0;             // work of the fullest CTA, summed over the launches of a step
 };
 
-static void deal_items(const spfm_batch *b, int policy, int depth, int slots, Deal &d)
+// deal false: only the span, by the mean, and the item count
+static void deal_items(const spfm_batch *b, int policy, int depth, int slots, bool deal, Deal &d)
 {
     constexpr int kStart = 3;   // halo planes and start of an item, in planes
     std::vector<BatchItem> list[2];
@@ -181,19 +183,46 @@ static void deal_items(const spfm_batch *b, int policy, int depth, int slots, De
     d.items.clear();
     d.starts.assign(2 * (kMaxCtas + 1), 0);
     d.span = 0;
+    if (!deal) {   // with many items a CTA the dealt work is the mean
+        for (int s = 0; s < 2; ++s) {
+            long long work = 0;
+            for (const BatchItem &i : list[s]) work += i.zc1 - i.zc0 + kStart;
+            if (d.ctas[s]) d.span += (work + d.ctas[s] - 1) / d.ctas[s];
+        }
+        d.count = list[0].size() + list[1].size();
+        return;
+    }
     for (int s = 0; s < 2; ++s) {
         std::vector<BatchItem> &l = list[s];
         const int ctas = d.ctas[s];
-        // longest first (stable: neighbouring tiles stay together), to the least loaded
-        std::stable_sort(l.begin(), l.end(), [](const BatchItem &x, const BatchItem &y) {
-            return x.zc1 - x.zc0 > y.zc1 - y.zc0;
-        });
+        // longest first (by counting, neighbouring tiles stay together)
+        {
+            std::vector<size_t> at(depth + 2, 0);
+            for (const BatchItem &i : l) ++at[depth - (i.zc1 - i.zc0) + 1];
+            for (int k = 0; k <= depth; ++k) at[k + 1] += at[k];
+            std::vector<BatchItem> sorted(l.size());
+            for (const BatchItem &i : l) sorted[at[depth - (i.zc1 - i.zc0)]++] = i;
+            l.swap(sorted);
+        }
         std::vector<int> owner(l.size()), count(ctas + 1, 0);
         std::priority_queue<std::pair<long long, int>, std::vector<std::pair<long long, int>>,
                             std::greater<std::pair<long long, int>>> least;
         for (int c = 0; c < ctas; ++c) least.push({0, c});
         long long span = 0;
-        for (size_t k = 0; k < l.size(); ++k) {
+        // to the least loaded; a long list in turn up to its last few rounds
+        const size_t turns = l.size() > 64u * (size_t)ctas ? (l.size() / ctas - 16) * ctas : 0;
+        if (turns) {
+            std::vector<long long> load(ctas, 0);
+            for (size_t k = 0; k < turns; ++k) {
+                const int c = (int)(k % ctas);
+                owner[k] = c;
+                ++count[c + 1];
+                load[c] += l[k].zc1 - l[k].zc0 + kStart;
+            }
+            least = decltype(least)();
+            for (int c = 0; c < ctas; ++c) least.push({load[c], c});
+        }
+        for (size_t k = turns; k < l.size(); ++k) {
             std::pair<long long, int> t = least.top();
             least.pop();
             owner[k] = t.second;
@@ -225,23 +254,22 @@ static cudaError_t set_depth(spfm_batch *b, int depth)
     Deal d;
     if (depth == 0) {
         long long best = -1;
-        Deal t;
         for (int p = 0; p < (b->dtype == SPFM_F32 ? 3 : 1); ++p)
             for (int c = kNDepths - 1; c >= 0; --c) {
-                const int policy = b->dtype == SPFM_F32 ? p : b->policy;
-                deal_items(b, policy, kDepths[c], slots, t);
-                const bool many = (long long)t.items.size() > 12LL * slots;
+                const int policy = b->dtype == SPFM_F32 ? p : SPFM_TILES_FIT;
+                Deal t;
+                deal_items(b, policy, kDepths[c], slots, false, t);
+                const bool many = t.count > 12u * (size_t)slots;
+                if (!many) deal_items(b, policy, kDepths[c], slots, true, t);
                 if (best < 0 || t.span < best || (t.span == best && b->policy == policy)) {
                     best = t.span;
                     depth = kDepths[c];
                     b->policy = policy;
-                    std::swap(d, t);
                 }
                 if (many) break;   // shorter items would only add halo planes
             }
-    } else {
-        deal_items(b, b->policy, depth, slots, d);
     }
+    deal_items(b, b->policy, depth, slots, true, d);
     b->depth = depth;
     b->nitems0 = d.nitems0;
     for (int s = 0; s < 2; ++s) b->ctas[s] = d.ctas[s];

@@ -15,9 +15,8 @@
 //
 // Boundary conditions.  The kernel reads the ghost layer.  In general it
 // writes interior cells only and a face kernel (boundary.cu) refreshes the
-// ghosts of the new field after each step.  When every
-// face is periodic and a row is a whole number of 32-byte sectors, the ghosts
-// are plain periodic images: the thread that writes a cell next to a face also
+// ghosts of the new field after each step.  When every face is periodic and a
+// row is a whole number of 32-byte sectors, the ghosts are plain periodic images: the thread that writes a cell next to a face also
 // writes its image(s) on the far side (x images as whole 32-byte sectors of
 // the row pads, two threads a sector), so no face kernel runs; where no face is
 // periodic the producer warp builds the ghosts of the planes it stages.  The
@@ -734,7 +733,8 @@ __device__ __noinline__ void call_sum_groups(const typename PackCoef<T>::Pair *p
 }
 
 // KIND: the potential (spfm_internal.h).  Degrees below the kernel's are padded
-// with zero coefficients, which changes no bit.
+// with zero coefficients, which changes no bit.  IMM: the coefficients PC are in
+// memory (a batch's), the constants 1, -2, -4 immediates.
 // One tile (bx, by) of planes zc0..zc1-1.  The stage ring continues across the
 // tiles a CTA processes: plane i of this tile is ring slot base + i.  The
 // producer waits for its copies in flight before returning when drain is set.
@@ -1383,7 +1383,7 @@ cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, 
     constexpr int R = sizeof(S) == 2 ? 1 : SPFM_ROWS_PER_THREAD;
     constexpr int NT1 = TileShape<S, T, TX, TY, 1>::NTHREADS;
     // programmatic dependent launch: the kernel may begin while the previous
-    // kernel in the stream runs; cfg.mode says which boxes wait (griddepcontrol)
+    // kernel in the stream runs (griddepcontrol.wait)
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
