@@ -1168,15 +1168,18 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
 
 // Resident CTAs per SM the register budget is sized for: three by default;
 // the single-grid FP32 kernels fit four (96 registers, no spills, 20 warps per
-// SM: 2 % faster for TI_<120>, 3-6 % for CF at 512^3), while FP64 and BF16
-// spill there, and the persistent batch kernel keeps three.
+// SM: 2 % faster for TI_<120>, 3-6 % for CF at 512^3), while FP64 spills
+// there, and the persistent batch kernel keeps three.
 template <class S> struct MinBlocks { static constexpr int value = SPFM_MIN_CTAS; };
 template <> struct MinBlocks<float> { static constexpr int value = 4; };
 
-// (the stochastic-rounding kernels and the potentials with the guard on q keep
-// three CTAs per SM: at four their registers spill; 150 x 133 x 117 with a
-// random normal 12.4 us a step at three, 12.6 at four, and the guard in the
-// kernels of 1 to 4 groups, which do not need it, cost 18 % at 512^3)
+// (The potentials with the guard on q keep three CTAs per SM: at four their
+// registers spill; 150 x 133 x 117 with a random normal 12.4 us a step at three,
+// 12.6 at four, and the guard in the kernels of 1 to 4 groups, which do not need
+// it, cost 18 % at 512^3.  The stochastic-rounding kernels keep three too: four
+// fit without spills and gain at the largest sizes, 512^3 TI 234.0 -> 233.0 us,
+// 256^3 CF contact 38.8 -> 35.8, but lose at the small ones, 128^3 7.8 -> 8.2,
+// 32^3 3.2 -> 3.5; BF16 likewise, 512^3 241 -> 235, 128^3 7.5 -> 7.9.)
 template <class S, class T, int STENCIL, int KIND, int TX, int TY, int RPT_, bool IMG, bool SR = false>
 __global__ void __launch_bounds__(TileShape<S, T, TX, TY, RPT_>::NTHREADS,
                                   KIND == kKindLocal ? 2 : ((SR || KIND > 4) ? SPFM_MIN_CTAS : MinBlocks<S>::value))
