@@ -814,7 +814,11 @@ __device__ __forceinline__ bool step_tile(const StepCoef<T> &C, const PackCoef<T
                     bulk_g2s(st + r * SW, plane + (long long)r * g.pitch, (uint32_t)bytes_row, &full[s]);
             }
         };
+        // The lanes' ghost stores precede, through ready, the consumers and empty, a
+        // later copy into the same stage by the asynchronous proxy, which the barriers
+        // alone do not order after stores of the generic proxy.
         auto release = [&](int j) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lead) mbar_arrive(&ready[(base + j) % NS]);
         };
