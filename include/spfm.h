@@ -169,6 +169,10 @@ int spfm_debug_pick_zchunk(int tiles, int nz, int per_sm, int sms, int target);
 int spfm_debug_potential(int dtype, int stencil, const double u[3], double lambda, double dx, int n,
                          const double *q, double *out, double *q_lo);
 
+/* Test hook (the paper has no counterpart): q[i] = a[i] / b[i] by the quotient
+ * of the FP64 step kernels, for n device arrays' elements on the stream. */
+spfm_status spfm_debug_quotient(int n, const double *a, const double *b, double *q, void *stream);
+
 /* Test hook of the failure reporting (the paper has no counterpart): the next
  * spfm_step launch skips the copy of one plane in its first CTA, whose bounded
  * waits (about 2 s each) then give up; the kernel returns without writing that

@@ -44,4 +44,20 @@ cudaError_t launch_batch_f64(const void *grids, BatchList list, int parity,
     return launch_batch_t<double, double, 16, 16>(grids, list, parity, err, stencil, kind, st, nullptr, 0,
                                                   fwd);
 }
+
+namespace {
+__global__ void quotient_kernel(int n, const double *a, const double *b, double *q)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        q[i] = Pk<double>::quot(a[i], b[i]);
+}
+}  // namespace
 }  // namespace spfm
+
+extern "C" spfm_status spfm_debug_quotient(int n, const double *a, const double *b, double *q, void *stream)
+{
+    if (n < 0 || !a || !b || !q) return SPFM_EINVAL;
+    if (n == 0) return SPFM_OK;
+    spfm::quotient_kernel<<<n / 256 + 1 < 1024 ? n / 256 + 1 : 1024, 256, 0, (cudaStream_t)stream>>>(n, a, b, q);
+    return cudaGetLastError() == cudaSuccess ? SPFM_OK : SPFM_ECUDA;
+}

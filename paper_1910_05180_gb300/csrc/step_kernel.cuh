@@ -104,18 +104,27 @@ template <> struct Pk<double> {
         return {__fma_rn(a.x, b.x, c.x), __fma_rn(a.y, b.y, c.y)};
     }
     static __device__ __forceinline__ P sub(P a, P b) { return {__dsub_rn(a.x, b.x), __dsub_rn(a.y, b.y)}; }
-    // a / b as a * r(b), r(b) the reciprocal by one third-order Newton step from
-    // the hardware's approximation (relative error e < 2^-18, then e^3): 5
-    // instructions of the FP64 pipe, which bounds these kernels, where a division
-    // takes some 14; within 2 ulp for |b| in the normal range, and a zero,
-    // infinite or NaN b gives a non-finite or zero result as the division does
+    // a / b in 7 instructions of the FP64 pipe, which bounds these kernels, where
+    // a division takes some 14: the reciprocal r by one third-order Newton step
+    // (Householder's iteration of order 2) from the hardware's approximation
+    // (relative error e < 2^-18, then e^3), and Markstein's correction of the
+    // quotient q by its remainder a - b q, which an FMA gives exactly (IBM J. Res.
+    // Dev. 34, 1990): correctly rounded but for quotients within 2^-50 ulp of a tie.
+    // The exponents of a and b keep the remainder and the reciprocal normal;
+    // other operands (zeros, infinities, NaN, far too large or small) are divided.
     static __device__ __forceinline__ double quot(double a, double b)
     {
+        constexpr uint32_t lo = (uint32_t)(1023 - 400) << 20, hi = (uint32_t)(1023 + 400) << 20;
+        const uint32_t ea = (uint32_t)__double2hiint(a) & 0x7fffffffu, eb = (uint32_t)__double2hiint(b) & 0x7fffffffu;
+        if (ea - lo >= hi - lo || eb - lo >= hi - lo) return divide(a, b);
         double r;
         asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
         const double e = __fma_rn(-b, r, 1.0);
-        return __dmul_rn(a, __fma_rn(__fma_rn(e, e, e), r, r));
+        r = __fma_rn(__fma_rn(e, e, e), r, r);
+        const double q = __dmul_rn(a, r);
+        return __fma_rn(__fma_rn(-b, q, a), r, q);
     }
+    static __device__ __noinline__ double divide(double a, double b) { return __ddiv_rn(a, b); }
     static __device__ __forceinline__ P div(P a, P b) { return {quot(a.x, b.x), quot(a.y, b.y)}; }
     static __device__ __forceinline__ P rsqrt(P a) { return {::rsqrt(a.x), ::rsqrt(a.y)}; }
     // v - v^2, rounded once
