@@ -72,9 +72,16 @@ __device__ __forceinline__ double corrected(double d, double x, double alpha, DF
 {
     return d - alpha * (x * (1.0 - x));
 }
-__device__ __forceinline__ float corrected(float d, float x, double, DF alpha)
+// alpha beyond the FP32 range (only minute cells take a correction then): as a
+// call, since inlined its FP64 instructions took a relaxation step 21.2 -> 25.7 us
+__device__ __noinline__ float corrected_wide(float d, float x, double alpha)
 {
-    const DF t = df_mul(alpha, q_of(x));
+    return (float)((double)d - alpha * ((double)x * (1.0 - (double)x)));
+}
+__device__ __forceinline__ float corrected(float d, float x, double alpha, DF alpha2)
+{
+    if (!isfinite(alpha2.lo)) return corrected_wide(d, x, alpha);
+    const DF t = df_mul(alpha2, q_of(x));
     const DF s = df_two_sum(d, -t.hi);
     return __fadd_rn(s.hi, __fsub_rn(s.lo, t.lo));
 }
