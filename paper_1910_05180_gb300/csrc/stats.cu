@@ -158,8 +158,8 @@ __device__ __forceinline__ void block_reduce_store(const double (&sum)[kSums], R
 //     the band test run in the storage precision, where they are exact (the
 //     band limits 1e-6 and 1 - 1e-6 are not floats, so the first float above
 //     and the last float below them decide exactly the same cells);
-//   - an FP32 field's volume is summed per lane and row as unevaluated pairs
-//     (TwoSum, Knuth TAOCP vol. 2, 4.2.2), two chains on the paired FP32
+//   - an FP32 field's volume is summed per lane and four sweeps as unevaluated
+//     pairs (TwoSum, Knuth TAOCP vol. 2, 4.2.2), two chains on the paired FP32
 //     instructions, carried in 2^-48 fixed point;
 //   - a row of cells is taken as finite and tested for band cells as a whole (a
 //     sum that is not finite has the lane look at its cells one by one; one
@@ -252,16 +252,20 @@ __device__ __forceinline__ long long fix48(float y)
     return (b >> 31) ? -v : v;
 }
 
-// Volume of one lane.  FP32 values: each row as an unevaluated pair s + c
-// (TwoSum) over four rows, then the pair in 2^-48 fixed point (exact to the
-// dropped bits, below 4e-15 per four rows), carried into FP64 before the fixed
-// point could overflow.
+// Volume of one lane.  FP32 values: unevaluated pairs s + c (TwoSum) over four
+// sweeps, that is 64 cells a lane, then the pair in 2^-48 fixed point, carried
+// into FP64 before the fixed point could overflow.  The sums s are exact but for
+// what c takes; c is an FP32 sum of up to 32 such remainders a chain: for cells in
+// [0, 1] each is at most 2^-20 and c at most 2^-15, so its roundings add up to
+// 32 * 2^-40 = 3e-11 at the very most per four sweeps, typically 1e-14 (random
+// profiles), beside the 2^-48 that the fixed point drops.  The count is of sweeps,
+// not of rows, so that the chains stay that short where a row has more than one.
 template <class R> struct VolSum;
 template <> struct VolSum<float> {
     float2 s = {0.0f, 0.0f}, c = {0.0f, 0.0f};   // two chains
     long long fix = 0;
     double sum = 0.0;
-    int rows = 0, flushes = 0;
+    int sweeps = 0, flushes = 0;
     static __device__ __forceinline__ float2 sub(float2 a, float2 b)
     {
         return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
@@ -280,12 +284,12 @@ template <> struct VolSum<float> {
         s = make_float2(r.x, r.y);
         c = make_float2(r.z, r.w);
     }
-    // the chains into fixed point (every fourth row: a row of 512 cells is 16 a lane)
+    // the chains into fixed point
     __device__ __forceinline__ void flush()
     {
         const DF t = df_two_sum(s.x, s.y);
         const float lo = (c.x + c.y) + t.lo;
-        if (fabsf(t.hi) < 256.0f) fix += fix48(t.hi) + fix48(lo);
+        if (fabsf(t.hi) < 256.0f && fabsf(lo) < 256.0f) fix += fix48(t.hi) + fix48(lo);
         else sum += (double)t.hi + (double)lo;
         set_row(make_float4(0.0f, 0.0f, 0.0f, 0.0f));
         if (++flushes == 32) {
@@ -294,9 +298,9 @@ template <> struct VolSum<float> {
             flushes = 0;
         }
     }
-    __device__ __forceinline__ void end_row()
+    __device__ __forceinline__ void end_sweep()
     {
-        if ((++rows & 3) == 0) flush();
+        if ((++sweeps & 3) == 0) flush();
     }
     __device__ __forceinline__ double total()
     {
@@ -308,7 +312,7 @@ template <> struct VolSum<double> {
     double sum = 0.0;
     __device__ __forceinline__ void add(double x) { sum += x; }
     __device__ __forceinline__ int row() const { return 0; }
-    __device__ __forceinline__ void end_row() {}
+    __device__ __forceinline__ void end_sweep() {}
     __device__ __forceinline__ double total() const { return sum; }
 };
 
@@ -620,8 +624,8 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
                     for (int k = 0; k + kW < 4 * V; ++k) u[k] = u[k + kW];
                 }
             }
+            vol.end_sweep();
         }
-        vol.end_row();
     }
     if (lane < tail - head) eval_at(head + lane);
     double energy = 0.0;
