@@ -121,17 +121,20 @@ int build_model(spfm_grid *g, double M, double Gamma, double lambda, double dx, 
     }
     m.rat.deg = 0;
     if (scheme == SPFM_TI_GLOBAL) {
-        // beta scales with D alone, so the grid's form at D = 1 serves every M
+        // the grid's form at sum beta = 1 serves every M and does not depend on the
+        // unit of length (beta goes with D / dx^2)
+        double total = 0.0;
+        for (int t = 0; t < m.nterms; ++t) total += m.beta[t];
         if (g->rat_lambda != lambda || g->rat_dx != dx || g->rat_stencil != stencil) {
             double b1[kMaxTerms];
-            for (int t = 0; t < m.nterms; ++t) b1[t] = m.beta[t] / m.D;
+            for (int t = 0; t < m.nterms; ++t) b1[t] = m.beta[t] / total;
             build_rational(m.A, m.E, b1, m.nterms, g->d.dtype != SPFM_F64, g->rat);
             g->rat_lambda = lambda;
             g->rat_dx = dx;
             g->rat_stencil = stencil;
         }
         m.rat = g->rat;
-        for (int i = 0; i < m.rat.deg; ++i) m.rat.num[i] *= m.D;
+        for (int i = 0; i < m.rat.deg; ++i) m.rat.num[i] *= total;
     }
     m.kmu = 4.0 * M * dF / (lambda * Gamma);
     m.kappa = m.D / (lambda * lambda) * (16.0 / 3.0) * wsum;

@@ -11,7 +11,7 @@ namespace spfm_host {
 
 // sum_k beta_k / (1 - A_k s^2) as N(q) / D(q) of q = phi (1 - phi): coefficients
 // of q^i (deg of them in N, deg + 1 in D, D(0) = 1), the lowest q it covers
-// (-inf: all).  deg 0: no such form within the FP32 range.
+// (-inf: all).  deg 0: no such form within the compute type's range.
 struct Rational {
     int deg = 0;
     double num[spfm::kMaxTerms], den[spfm::kMaxTerms + 1], q_lo;
@@ -38,7 +38,7 @@ struct spfm_grid {
     bool skip_copy = false;   // spfm_debug_skip_copy: the next step launch skips one copy
     int zchunk = 0;           // spfm_set_zchunk: planes per CTA of the step launches (0: chosen per launch)
     int last_zchunk = 0;      // planes per CTA of the last step launch
-    // N / D of the TI potential for these lambda, dx and stencil, at D = 1
+    // N / D of the TI potential for these lambda, dx and stencil, at sum beta = 1
     // (build_model scales it); the groups follow from the descriptor's u, n and gamma
     spfm_host::Rational rat;
     double rat_lambda = 0.0, rat_dx = 0.0;
@@ -59,9 +59,9 @@ int check_extent(const spfm_grid_desc *d, size_t pitch_x, const char *who);
 
 // Model coefficients in FP64 (a1).  gamma defaults, nu_j = 3/m_j, c_j, A_k
 // grouped by value, stability and phase checks.
-// From K groups with A_k, E_k = 1 - A_k and beta_k (potential.cu).  fewer: as
-// few terms as keep the sum to 2^-30 (FP32 compute); else all K.
-void build_rational(const double *A, const double *E, const double *beta, int K, bool fewer, Rational &r);
+// From K groups with A_k, E_k = 1 - A_k and beta_k of sum 1 (potential.cu).  fp32:
+// as few terms as keep the sum to 2^-30, coefficients in the FP32 range; else all K.
+void build_rational(const double *A, const double *E, const double *beta, int K, bool fp32, Rational &r);
 
 struct Model {
     double gamma[3], w[spfm::kMaxTerms], c_shell[3], ck[spfm::kMaxTerms];

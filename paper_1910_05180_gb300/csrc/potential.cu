@@ -36,7 +36,8 @@ namespace {
 
 constexpr int kK = spfm::kMaxTerms;
 constexpr double kTol = 0x1p-30;
-constexpr double kMaxCoef = 1e24;   // FP32 range of the coefficients, with room for q outside [0, 1/4]
+// largest coefficients, with room for q outside [0, 1/4] in the compute type's range
+constexpr double kMaxCoef32 = 1e24, kMaxCoef64 = 1e100;
 
 // Eigenvalues d and first components z of the unit eigenvectors of the n x n
 // symmetric tridiagonal matrix with diagonal d and off-diagonal e, by QL
@@ -118,8 +119,8 @@ bool reduce(const double *A, const double *beta, int K, int N, const double *u, 
     return true;
 }
 
-// N(q) / D(q) of the nodes x with e = 1 - x and weights w; false outside kMaxCoef
-bool expand(const double *x, const double *e, const double *w, int N, Rational &r)
+// N(q) / D(q) of the nodes x with e = 1 - x and weights w; false above max_coef
+bool expand(const double *x, const double *e, const double *w, int N, double max_coef, Rational &r)
 {
     r.deg = N;
     for (int i = 0; i < kK; ++i) r.num[i] = 0.0;
@@ -131,22 +132,23 @@ bool expand(const double *x, const double *e, const double *w, int N, Rational &
         for (int i = k + 1; i >= 1; --i) r.den[i] += g * r.den[i - 1];
     }
     for (int i = 0; i <= N; ++i)
-        if (!(r.den[i] < kMaxCoef) || (i < N && !(r.num[i] < kMaxCoef))) return false;
+        if (!(r.den[i] < max_coef) || (i < N && !(r.num[i] < max_coef))) return false;
     return true;
 }
 
 }  // namespace
 
-void build_rational(const double *A, const double *E, const double *beta, int K, bool fewer, Rational &r)
+void build_rational(const double *A, const double *E, const double *beta, int K, bool fp32, Rational &r)
 {
+    const double max_coef = fp32 ? kMaxCoef32 : kMaxCoef64;
     r.deg = 0;
     r.q_lo = -HUGE_VAL;
     if (K < 1) {   // no coupled direction: the sum is 0
         const double x = 0.0, e = 1.0, w = 0.0;
-        expand(&x, &e, &w, 1, r);
+        expand(&x, &e, &w, 1, max_coef, r);
         return;
     }
-    if (fewer && K > 2) {
+    if (fp32 && K > 2) {
         double amax = 0.0;
         for (int k = 0; k < K; ++k) amax = std::max(amax, A[k]);
         const double pole = 1.0 / amax, u_hi = 1.0 + std::min(0.05, 0.25 * (pole - 1.0));
@@ -168,13 +170,13 @@ void build_rational(const double *A, const double *E, const double *beta, int K,
             }
             if (!(worst < kTol)) continue;
             for (int j = 0; j < N; ++j) e[j] = 1.0 - x[j];
-            if (expand(x, e, w, N, r)) {
+            if (expand(x, e, w, N, max_coef, r)) {
                 r.q_lo = 0.25 * (1.0 - u_hi);
                 return;
             }
         }
     }
-    if (!expand(A, E, beta, K, r)) r.deg = 0;
+    if (!expand(A, E, beta, K, max_coef, r)) r.deg = 0;
 }
 
 }  // namespace spfm_host
