@@ -152,9 +152,10 @@ void build_rational(const double *A, const double *E, const double *beta, int K,
         double amax = 0.0;
         for (int k = 0; k < K; ++k) amax = std::max(amax, A[k]);
         const double pole = 1.0 / amax, u_hi = 1.0 + std::min(0.05, 0.25 * (pole - 1.0));
-        const double l0 = log(pole), l1 = log(pole - u_hi);
+        const bool room = pole - u_hi > 0.0;   // none where some A_k is 1
+        const double l0 = log(pole), l1 = room ? log(pole - u_hi) : l0;
         // a generic normal needs about 2.7 + log(pole / (pole - u_hi)) terms: the search starts there
-        for (int N = std::max(2, (int)(2.7 + l0 - l1)); N < K && pole - u_hi > 0.0; ++N) {
+        for (int N = std::max(2, (int)(2.7 + l0 - l1)); N < K && room; ++N) {
             double u[2 * kK], x[kK], w[kK], e[kK];
             for (int i = 0; i < 2 * N; ++i)
                 u[i] = pole - exp(l0 + (l1 - l0) * 0.5 * (1.0 - cos(M_PI * (2 * i + 1) / (4.0 * N))));
