@@ -156,7 +156,14 @@ int spfm_last_zchunk(const spfm_grid *g);
 /* Test hook (the paper has no counterpart): the chunk length the automatic
  * choice gives a launch of `tiles` xy tiles over nz planes, for a kernel of
  * per_sm resident CTAs per SM on sms SMs, with `target` CTAs for grids of many
- * rounds.  Host only, no device call.  -1 for an argument below 1. */
+ * rounds; family 0: the FP32 and BF16 kernels of the TI and CF potentials, 1: TI_n,
+ * 2: the FP64 kernels of the TI and CF potentials.  Host only, no device call.
+ * -1 for an unknown family or another argument below 1. */
+int spfm_debug_zchunk(int family, int tiles, int nz, int per_sm, int sms, int target);
+
+/* Test hook (the paper has no counterpart): the dispatch model of family 0
+ * alone, which the choice follows for launches of more than one round of
+ * 4-plane chunks; arguments and errors as above. */
 int spfm_debug_pick_zchunk(int tiles, int nz, int per_sm, int sms, int target);
 
 /* Test hook (the paper has no counterpart): the TI potential's sum over the

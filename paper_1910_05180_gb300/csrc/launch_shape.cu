@@ -43,7 +43,7 @@
 // The FP64 kernels (CF and TI global) are bound by the FP64 pipe, which the CTAs
 // of an SM share: what counts is the work of the fullest SM, ceil(CTAs / SMs)
 // CTAs, a plane of a CTA costing about 9 FP64 instructions a cell as it is read
-// and 18 more as it is written (the halo planes are only read).  A CTA alone on
+// and 21 more as it is written (the halo planes are only read).  A CTA alone on
 // its SM leaves the pipe idle a fifth of the time, two leave it 2 %.  Chunks of
 // 1 to 64 planes, the least work, ties to the longer chunk.  Measured, us a step
 // (planes per CTA): 128 x 32 x 32 7-point 2 (chosen) 10.6, 1: 15.0, 4 (the
@@ -134,13 +134,22 @@ static int fp64_zchunk(int tiles, int nz, int sms)
     for (int zc = 1; zc <= (nz < 64 ? nz : 64); ++zc) {
         const long long ctas = (long long)tiles * ((nz + zc - 1) / zc);
         const long long n = (ctas + sms - 1) / sms, idle = n == 1 ? 20 : (n == 2 ? 2 : 0);
-        const long long work = n * (100 + idle) * (9 * (zc + 2) + 18 * zc);
+        const long long work = n * (100 + idle) * (9 * (zc + 2) + 21 * zc);
         if (best_work < 0 || work <= best_work) {
             best_work = work;
             best = zc;
         }
     }
     return best;
+}
+
+int choose_zchunk(int family, int tiles, int nz, int per_sm, int sms, int target)
+{
+    const int slots = per_sm * sms;
+    if (family == kUneven) return uneven_zchunk(tiles, nz, slots);
+    if (family == kFp64) return fp64_zchunk(tiles, nz, sms);
+    if ((long long)tiles * ((nz + 3) / 4) <= slots) return one_round_zchunk(tiles, nz, slots);
+    return model_zchunk(tiles, nz, per_sm, slots, target);
 }
 
 namespace {
@@ -174,10 +183,7 @@ int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target, in
     auto z = g_zc.find(zk);
     if (z != g_zc.end()) return z->second;
     if (g_zc.size() >= 4096) g_zc.clear();   // many grid shapes (a serving process): start over
-    const int zc = family == kUneven ? uneven_zchunk(tiles, nz, slots)
-                   : family == kFp64 ? fp64_zchunk(tiles, nz, sms)
-                   : (long long)tiles * ((nz + 3) / 4) <= slots ? one_round_zchunk(tiles, nz, slots)
-                                                                : model_zchunk(tiles, nz, per_sm, slots, target);
+    const int zc = choose_zchunk(family, tiles, nz, per_sm, sms, target);
     g_zc[zk] = zc;
     return zc;
 }
@@ -188,4 +194,11 @@ extern "C" int spfm_debug_pick_zchunk(int tiles, int nz, int per_sm, int sms, in
 {
     if (tiles < 1 || nz < 1 || per_sm < 1 || sms < 1 || target < 1) return -1;
     return spfm::model_zchunk(tiles, nz, per_sm, per_sm * sms, target);
+}
+
+extern "C" int spfm_debug_zchunk(int family, int tiles, int nz, int per_sm, int sms, int target)
+{
+    if (family < spfm::kStream || family > spfm::kFp64) return -1;
+    if (tiles < 1 || nz < 1 || per_sm < 1 || sms < 1 || target < 1) return -1;
+    return spfm::choose_zchunk(family, tiles, nz, per_sm, sms, target);
 }

@@ -198,6 +198,8 @@ struct LaunchCfg {
 // kStream).  Cached per kernel and shape.
 enum { kStream = 0, kUneven = 1, kFp64 = 2 };
 int pick_zchunk(const void *kern, int threads, int tiles, int nz, int target, int family);
+// The same for a kernel of per_sm resident CTAs per SM on sms SMs (host arithmetic alone).
+int choose_zchunk(int family, int tiles, int nz, int per_sm, int sms, int target);
 
 // How a step launch runs.  Launches chain by programmatic dependent launch: every
 // kernel of a call may start while the one before runs and waits for the whole of

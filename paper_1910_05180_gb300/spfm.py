@@ -98,6 +98,7 @@ SIGNATURES = [
     ("spfm_set_zchunk", _I, [_P, _I]),
     ("spfm_last_zchunk", _I, [_P]),
     ("spfm_debug_pick_zchunk", _I, [_I, _I, _I, _I, _I]),
+    ("spfm_debug_zchunk", _I, [_I, _I, _I, _I, _I, _I]),
     ("spfm_debug_potential", _I, [_I, _I, ctypes.POINTER(_D), _D, _D, _I, ctypes.POINTER(_D), ctypes.POINTER(_D),
                                   ctypes.POINTER(_D)]),
     ("spfm_debug_quotient", _I, [_I, _P, _P, _P, _P]),
