@@ -176,6 +176,13 @@ int spfm_debug_pick_zchunk(int tiles, int nz, int per_sm, int sms, int target);
 int spfm_debug_potential(int dtype, int stencil, const double u[3], double lambda, double dx, int n,
                          const double *q, double *out, double *q_lo);
 
+/* Test hook (the paper has no counterpart): the CTA that each of n batch items of
+ * planes[i] planes goes to when they are dealt to ctas CTAs (owner), and the
+ * work of the fullest one by the rule without turns (span, may be NULL; an item's
+ * work is its planes + 3).  Host only, no device call.  0, or -1 for bad
+ * arguments. */
+int spfm_debug_deal(int n, const int *planes, int ctas, int *owner, long long *span);
+
 /* Test hook (the paper has no counterpart): q[i] = a[i] / b[i] by the quotient
  * of the FP64 step kernels, for n device arrays' elements on the stream. */
 spfm_status spfm_debug_quotient(int n, const double *a, const double *b, double *q, void *stream);

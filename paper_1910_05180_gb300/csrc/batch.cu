@@ -23,8 +23,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <queue>
-#include <utility>
 #include <vector>
 
 #include "host_internal.h"
@@ -161,14 +159,10 @@ struct Deal {
     std::vector<BatchItem> items;   // in CTA order, shape 0 first
     std::vector<int> starts;        // kMaxCtas + 1 entries a shape
     int ctas[2] = {0, 0}, nitems0 = 0;
-    size_t count = 0;               // items
-    long long span = 0;             // work of the fullest CTA, summed over the launches of a step
 };
 
-// deal false: only the span, by the mean, and the item count
-static void deal_items(const spfm_batch *b, int policy, int depth, int slots, bool deal, Deal &d)
+static void deal_items(const spfm_batch *b, int policy, int depth, int slots, Deal &d)
 {
-    constexpr int kStart = 3;   // halo planes and start of an item, in planes
     std::vector<BatchItem> list[2];
     for (int i = 0; i < b->n; ++i) {
         const GridGeom &g = b->grids[i]->geom;
@@ -178,68 +172,47 @@ static void deal_items(const spfm_batch *b, int policy, int depth, int slots, bo
         l.resize(at + items_of(b->dtype, g, i, depth, nullptr, shape));
         items_of(b->dtype, g, i, depth, l.data() + at, shape);
     }
-    slots = std::min(slots, kMaxCtas);
-    for (int s = 0; s < 2; ++s) d.ctas[s] = (int)std::min<size_t>(list[s].size(), slots);
-    d.items.clear();
     d.starts.assign(2 * (kMaxCtas + 1), 0);
-    d.span = 0;
-    if (!deal) {   // with many items a CTA the dealt work is the mean
-        for (int s = 0; s < 2; ++s) {
-            long long work = 0;
-            for (const BatchItem &i : list[s]) work += i.zc1 - i.zc0 + kStart;
-            if (d.ctas[s]) d.span += (work + d.ctas[s] - 1) / d.ctas[s];
-        }
-        d.count = list[0].size() + list[1].size();
-        return;
-    }
     for (int s = 0; s < 2; ++s) {
-        std::vector<BatchItem> &l = list[s];
-        const int ctas = d.ctas[s];
-        // longest first (by counting, neighbouring tiles stay together)
-        {
-            std::vector<size_t> at(depth + 2, 0);
-            for (const BatchItem &i : l) ++at[depth - (i.zc1 - i.zc0) + 1];
-            for (int k = 0; k <= depth; ++k) at[k + 1] += at[k];
-            std::vector<BatchItem> sorted(l.size());
-            for (const BatchItem &i : l) sorted[at[depth - (i.zc1 - i.zc0)]++] = i;
-            l.swap(sorted);
-        }
-        std::vector<int> owner(l.size()), count(ctas + 1, 0);
-        std::priority_queue<std::pair<long long, int>, std::vector<std::pair<long long, int>>,
-                            std::greater<std::pair<long long, int>>> least;
-        for (int c = 0; c < ctas; ++c) least.push({0, c});
-        long long span = 0;
-        // to the least loaded; a long list in turn up to its last few rounds
-        const size_t turns = l.size() > 64u * (size_t)ctas ? (l.size() / ctas - 16) * ctas : 0;
-        if (turns) {
-            std::vector<long long> load(ctas, 0);
-            for (size_t k = 0; k < turns; ++k) {
-                const int c = (int)(k % ctas);
-                owner[k] = c;
-                ++count[c + 1];
-                load[c] += l[k].zc1 - l[k].zc0 + kStart;
-            }
-            least = decltype(least)();
-            for (int c = 0; c < ctas; ++c) least.push({load[c], c});
-        }
-        for (size_t k = turns; k < l.size(); ++k) {
-            std::pair<long long, int> t = least.top();
-            least.pop();
-            owner[k] = t.second;
-            ++count[t.second + 1];
-            t.first += l[k].zc1 - l[k].zc0 + kStart;
-            span = std::max(span, t.first);
-            least.push(t);
-        }
+        const std::vector<BatchItem> &l = list[s];
+        const int ctas = d.ctas[s] = (int)std::min<size_t>(l.size(), slots);
+        std::vector<int> planes(l.size()), order, owner, next(ctas + 1, 0);
+        for (size_t k = 0; k < l.size(); ++k) planes[k] = l[k].zc1 - l[k].zc0;
+        deal(planes, ctas, order, owner);
         int *start = d.starts.data() + s * (kMaxCtas + 1);
-        for (int c = 0; c < ctas; ++c) start[c + 1] = start[c] + count[c + 1];
+        for (int o : owner) ++next[o + 1];
+        for (int c = 0; c < ctas; ++c) start[c + 1] = next[c + 1] += next[c];
         const size_t at = d.items.size();
         d.items.resize(at + l.size());
-        std::vector<int> next(start, start + ctas);
-        for (size_t k = 0; k < l.size(); ++k) d.items[at + next[owner[k]]++] = l[k];
+        for (size_t k = 0; k < l.size(); ++k) d.items[at + next[owner[k]]++] = l[order[k]];
         if (s == 0) d.nitems0 = (int)l.size();
-        d.span += span;
     }
+}
+
+// The work of the fullest CTA, summed over the launches of a step, of a tile policy
+// and depth; with many items a slot (*many) by the mean, which the deal comes to
+// then.  Counted by length, without the items: dealt for every candidate, creating
+// a batch of 64 grids of 32 to 96 cells took 1.46 ms, so 0.15.
+static long long span_of(const spfm_batch *b, int policy, int depth, int slots, bool *many)
+{
+    std::vector<long long> count[2];
+    long long n[2] = {0, 0}, work[2] = {0, 0}, span = 0;
+    for (int s = 0; s < 2; ++s) count[s].assign(depth + 1, 0);
+    for (int i = 0; i < b->n; ++i) {
+        const GridGeom &g = b->grids[i]->geom;
+        const int shape = shape_for(b->dtype, g, policy), chunks = (g.nz + depth - 1) / depth;
+        const long long tiles = items_of(b->dtype, g, i, depth, nullptr, shape) / chunks;
+        count[shape][depth] += tiles * (g.nz / depth);
+        if (g.nz % depth) count[shape][g.nz % depth] += tiles;
+        n[shape] += tiles * chunks;
+        work[shape] += tiles * (g.nz + (long long)kItemStart * chunks);
+    }
+    *many = n[0] + n[1] > 12LL * slots;
+    for (int s = 0; s < 2; ++s) {
+        const int ctas = (int)std::min<long long>(n[s], slots);
+        if (ctas) span += *many ? (work[s] + ctas - 1) / ctas : deal_span(count[s], ctas);
+    }
+    return span;
 }
 
 // The work-list of z-march depth `depth` under the batch's tile policy (0: the
@@ -250,26 +223,25 @@ static cudaError_t set_depth(spfm_batch *b, int depth)
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int slots = b->slots = sms * kBatchCtasPerSm;
-    Deal d;
+    b->slots = sms * kBatchCtasPerSm;
+    const int slots = std::min(b->slots, kMaxCtas);
     if (depth == 0) {
         long long best = -1;
         for (int p = 0; p < (b->dtype == SPFM_F32 ? 3 : 1); ++p)
             for (int c = kNDepths - 1; c >= 0; --c) {
                 const int policy = b->dtype == SPFM_F32 ? p : SPFM_TILES_FIT;
-                Deal t;
-                deal_items(b, policy, kDepths[c], slots, false, t);
-                const bool many = t.count > 12u * (size_t)slots;
-                if (!many) deal_items(b, policy, kDepths[c], slots, true, t);
-                if (best < 0 || t.span < best || (t.span == best && b->policy == policy)) {
-                    best = t.span;
+                bool many;
+                const long long span = span_of(b, policy, kDepths[c], slots, &many);
+                if (best < 0 || span < best || (span == best && b->policy == policy)) {
+                    best = span;
                     depth = kDepths[c];
                     b->policy = policy;
                 }
                 if (many) break;   // shorter items would only add halo planes
             }
     }
-    deal_items(b, b->policy, depth, slots, true, d);
+    Deal d;
+    deal_items(b, b->policy, depth, slots, d);
     b->depth = depth;
     b->nitems0 = d.nitems0;
     for (int s = 0; s < 2; ++s) b->ctas[s] = d.ctas[s];

@@ -4,6 +4,7 @@
 #pragma once
 
 #include <string>
+#include <vector>
 
 #include "spfm_internal.h"
 
@@ -62,6 +63,16 @@ int check_extent(const spfm_grid_desc *d, size_t pitch_x, const char *who);
 // From K groups with A_k, E_k = 1 - A_k and beta_k of sum 1 (potential.cu).  fp32:
 // as few terms as keep the sum to 2^-30, coefficients in the FP32 range; else all K.
 void build_rational(const double *A, const double *E, const double *beta, int K, bool fp32, Rational &r);
+
+// Deal of a batch's items to CTAs (deal.cu).  An item costs its planes and
+// kItemStart more: two halo planes and its start.
+constexpr int kItemStart = 3;
+// order: the items longest first; owner[k]: the CTA of item order[k], the least
+// loaded so far (lists above 64 items a CTA: in turn up to the last rounds)
+void deal(const std::vector<int> &planes, int ctas, std::vector<int> &order, std::vector<int> &owner);
+// the work of the fullest CTA by that rule (each to the least loaded), for
+// count[p] items of p planes
+long long deal_span(const std::vector<long long> &count, int ctas);
 
 struct Model {
     double gamma[3], w[spfm::kMaxTerms], c_shell[3], ck[spfm::kMaxTerms];
