@@ -338,6 +338,9 @@ spfm_status spfm_batch_autotune(spfm_batch *b, const spfm_step_args *args, int s
 spfm_status spfm_batch_set_tiles(spfm_batch *b, int policy);
 /* The batch's current tile policy and z-march depth (either may be NULL). */
 spfm_status spfm_batch_tiles(const spfm_batch *b, int *policy, int *depth);
+/* Test hook (the paper has no counterpart): CUDA graphs the batch has captured so
+ * far (-1 for NULL). */
+int spfm_debug_batch_captures(const spfm_batch *b);
 /* Diagnostics of every grid in one pass; out has n entries.  Synchronises. */
 spfm_status spfm_batch_stats(spfm_batch *b, int flags, spfm_stats *out);
 spfm_status spfm_batch_destroy(spfm_batch *b);

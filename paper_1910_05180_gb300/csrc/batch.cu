@@ -33,6 +33,7 @@ using namespace spfm_host;
 namespace {
 
 constexpr int kGraphSteps = 16;    // steps per captured graph (even: parity repeats)
+constexpr size_t kGraphs = 4;      // captured graphs a batch keeps
 // depths the autotuner tries; the scratch holds the work-list of the shallowest
 constexpr int kDepths[] = {8, 12, 16, 24, 32, 48, 64};
 constexpr int kNDepths = (int)(sizeof(kDepths) / sizeof(kDepths[0]));
@@ -139,12 +140,23 @@ struct spfm_batch {
     // no grid has a periodic face: the step kernels compute the ghosts as they
     // read them and no ghost kernel runs between steps
     bool inline_faces = false;
-    cudaGraphExec_t exec = nullptr;
-    int graph_stencil = -1, graph_kind = -1, graph_sr = -1;
+    // Captured steps, the last used first: one for each kernel the calls take (the
+    // kind goes with the parameters of a call, which may alternate), at most kGraphs.
+    struct Graph {
+        cudaGraphExec_t exec;
+        int stencil, kind, sr;
+    };
+    std::vector<Graph> graphs;
+    int captures = 0;         // graphs captured so far
     std::string err;
     ~spfm_batch()
     {
-        if (exec) cudaGraphExecDestroy(exec);
+        drop_graphs();
+    }
+    void drop_graphs()
+    {
+        for (Graph &g : graphs) cudaGraphExecDestroy(g.exec);
+        graphs.clear();
     }
 };
 
@@ -247,10 +259,7 @@ static cudaError_t set_depth(spfm_batch *b, int depth)
     for (int s = 0; s < 2; ++s) b->ctas[s] = d.ctas[s];
     b->h_items.swap(d.items);
     b->h_starts.swap(d.starts);
-    if (b->exec) {
-        cudaGraphExecDestroy(b->exec);
-        b->exec = nullptr;
-    }
+    b->drop_graphs();
     cudaError_t e = cudaMemcpyAsync(b->scratch + b->L.items, b->h_items.data(), sizeof(BatchItem) * b->h_items.size(),
                                     cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess)
@@ -294,13 +303,15 @@ static cudaError_t launch_steps(spfm_batch *b, int first, int n, int stencil, in
     return e;
 }
 
+// the graph of kGraphSteps steps of these kernels, captured if need be, at the front of b->graphs
 static cudaError_t capture_graph(spfm_batch *b, int stencil, int kind)
 {
-    if (b->exec && b->graph_stencil == stencil && b->graph_kind == kind && b->graph_sr == b->sr) return cudaSuccess;
-    if (b->exec) {
-        cudaGraphExecDestroy(b->exec);
-        b->exec = nullptr;
-    }
+    std::vector<spfm_batch::Graph> &gs = b->graphs;
+    for (size_t i = 0; i < gs.size(); ++i)
+        if (gs[i].stencil == stencil && gs[i].kind == kind && gs[i].sr == b->sr) {
+            std::rotate(gs.begin(), gs.begin() + i, gs.begin() + i + 1);
+            return cudaSuccess;
+        }
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
@@ -309,15 +320,16 @@ static cudaError_t capture_graph(spfm_batch *b, int stencil, int kind)
         le = launch_advance_steps((long long *)(b->scratch + b->L.steps), b->n, kGraphSteps, b->stream);
     e = cudaStreamEndCapture(b->stream, &graph);
     if (le != cudaSuccess) e = le;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, graph, 0);
+    cudaGraphExec_t exec = nullptr;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
     if (graph) cudaGraphDestroy(graph);
-    if (e == cudaSuccess) {
-        b->graph_stencil = stencil;
-        b->graph_kind = kind;
-        b->graph_sr = b->sr;
-    } else {
-        b->exec = nullptr;
+    if (e != cudaSuccess) return e;
+    if (gs.size() == kGraphs) {
+        cudaGraphExecDestroy(gs.back().exec);
+        gs.pop_back();
     }
+    gs.insert(gs.begin(), {exec, stencil, kind, b->sr});
+    ++b->captures;
     return e;
 }
 
@@ -452,7 +464,7 @@ spfm_status spfm_batch_step(spfm_batch *b, int n_steps, const spfm_step_args *ar
         e = capture_graph(b, stencil, kind);
         if (e != cudaSuccess) return bfail(b, SPFM_ECUDA, cudaGetErrorString(e));
         for (; s + kGraphSteps <= n_steps; s += kGraphSteps) {
-            e = cudaGraphLaunch(b->exec, b->stream);
+            e = cudaGraphLaunch(b->graphs.front().exec, b->stream);
             if (e != cudaSuccess) return bfail(b, SPFM_ECUDA, cudaGetErrorString(e));
         }
     }
@@ -581,6 +593,8 @@ spfm_status spfm_batch_tiles(const spfm_batch *b, int *policy, int *depth)
     if (depth) *depth = b->depth;
     return SPFM_OK;
 }
+
+int spfm_debug_batch_captures(const spfm_batch *b) { return b ? b->captures : -1; }
 
 spfm_status spfm_batch_stats(spfm_batch *b, int flags, spfm_stats *out)
 {

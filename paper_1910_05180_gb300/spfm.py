@@ -101,6 +101,7 @@ SIGNATURES = [
     ("spfm_debug_zchunk", _I, [_I, _I, _I, _I, _I, _I]),
     ("spfm_debug_potential", _I, [_I, _I, ctypes.POINTER(_D), _D, _D, _I, ctypes.POINTER(_D), ctypes.POINTER(_D),
                                   ctypes.POINTER(_D)]),
+    ("spfm_debug_batch_captures", _I, [_P]),
     ("spfm_debug_deal", _I, [_I, ctypes.POINTER(_I), _I, ctypes.POINTER(_I), ctypes.POINTER(ctypes.c_longlong)]),
     ("spfm_debug_quotient", _I, [_I, _P, _P, _P, _P]),
     ("spfm_shift_x", _I, [_P, _I]),
