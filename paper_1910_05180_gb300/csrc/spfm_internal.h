@@ -205,10 +205,11 @@ int choose_zchunk(int family, int tiles, int nz, int per_sm, int sms, int target
 // kernel of a call may start while the one before runs and waits for the whole of
 // it before it reads.  When a kernel lets the next one start matters for balance:
 // CTAs that arrive early take the slots that happen to be free and crowd some
-// SMs, so a launch of few rounds does so at its end (us a step, start -> end:
-// 64^3 periodic TI_<111> 4.2 -> 3.3, 150 x 133 x 117 contact 11.3 -> 10.7, 64^3 FP64
-// 38.0 -> 24.7), while many rounds (kEarly) fill the slots that their tail leaves
-// (320^3 TI_n 155.3 -> 154.1).
+// SMs, so a launch of few CTAs does so as its own CTAs end (ends_launch in
+// step_kernel.cuh; us a step, start -> end: 64^3 periodic TI_<111> 4.2 -> 3.3, 150 x
+// 133 x 117 contact 11.3 -> 10.7), while a launch of many (kEarly: four times the
+// design occupancy of its storage type, 16 CTAs an SM in FP32 and 12 in BF16 and
+// FP64) fills the slots that its tail leaves (320^3 TI_n 155.3 -> 154.1).
 //   kImages     all faces periodic: the step writes the ghost images of its new cells
 //               itself (no face kernel follows)
 //   kSkipCopy   test of the bounded waits: the first CTA skips one plane's copy

@@ -740,6 +740,20 @@ __device__ __noinline__ void call_sum_groups(const typename PackCoef<T>::Pair *p
     sum_groups<T>(pair, n, u, num, den);
 }
 
+// Whether this thread lets the next launch start at the end of its CTA: the first
+// thread of a CTA that triggers counts.  A consumer, after its last plane, since
+// the producer warp ends up to a ring of planes before it (us a step, trigger by
+// the warp that ends first -> by a consumer: FP64 96^3 periodic 142 -> 95, contact
+// 158 -> 112; FP32 64^3 periodic 3.6 -> 3.1, 128^3 channel 8.5 -> 8.0).  In FP32 and
+// BF16 grids whose ghosts the producer builds the planes are released one by
+// one, and there the warp that ends first is as good or better (64^3 contact 4.79
+// against 4.88, 96^3 7.04 against 7.28).
+template <class T>
+__device__ __forceinline__ bool ends_launch(bool fwd)
+{
+    return (fwd && sizeof(T) == 4) || threadIdx.x == 0;
+}
+
 // KIND: the potential (spfm_internal.h).  Degrees below the kernel's are padded
 // with zero coefficients, which changes no bit.  IMM: the coefficients PC are in
 // memory (a batch's), the constants 1, -2, -4 immediates.
@@ -1224,7 +1238,7 @@ __global__ void __launch_bounds__(TileShape<S, T, TX, TY, RPT_>::NTHREADS,
     step_tile<S, T, STENCIL, KIND, TX, TY, RPT_, IMG, SR>(C, PC, src, dst, err, use_tmap ? &tmap : nullptr,
                                                      blockIdx.x, blockIdx.y, zc0, zc1, stages, full, empty, 0,
                                                      true, mode, C.sr_key, ready, fwd, true);
-    if (!(mode & kEarly)) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!(mode & kEarly) && ends_launch<T>(fwd)) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // ------------------------------------------------------------------- batches
@@ -1301,7 +1315,7 @@ __global__ void __launch_bounds__(TileShape<S, T, TX, TY>::NTHREADS, kBatchCtasP
             return;
         base += it.zc1 - it.zc0 + 2;
     }
-    if (!list.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!list.early && ends_launch<T>(fwd != 0)) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Work-list entries of one grid for the tile shape (TX, TY) of the (S, T)
