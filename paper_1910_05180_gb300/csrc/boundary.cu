@@ -75,7 +75,9 @@ __global__ void __launch_bounds__(256) ghost_kernel(const FaceArgs a, S *f)
     // May launch while the step before it runs, and lets the next step launch when
     // its blocks are through: launched earlier, that one's CTAs take the slots that
     // happen to be free and crowd some SMs (us a step, trigger at the start of this
-    // kernel -> here: 96^3 FP64 82.4 -> 56.3, 128^3 FP32 9.6 -> 8.5).
+    // kernel -> here: 96^3 FP64 82.4 -> 56.3, 128^3 FP32 9.6 -> 8.5, 256^3 30.9 -> 30.1,
+    // 384^3 88.7 -> 88.5, 512^3 187.8 -> 187.5; with interior tiles of the next step
+    // that do not wait for this kernel at all: 256^3 33.5, 384^3 89.3, 512^3 188.4).
     asm volatile("griddepcontrol.wait;" ::: "memory");
     ghost_faces<S>(a, f, blockIdx.x * (long long)blockDim.x + threadIdx.x,
                    (long long)gridDim.x * blockDim.x);

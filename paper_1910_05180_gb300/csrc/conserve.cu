@@ -171,8 +171,8 @@ __device__ __forceinline__ int axis_image(int m, int c, int n, bool periodic)
 // E cells (i.., j, k) of a row with their stored values v, and the ghosts they
 // are the source of, as the face kernel (boundary.cu) writes them: shifts along
 // x, then y, then z in the compute type (CONTACT: some face has the shift of
-// Eq. 7; without it the images are copies: 4 us less at 60^3).  The y and z images are the warp's, whole rows at a time; most rows
-// have none.
+// Eq. 7; without it the images are copies: 4 us less at 60^3).  The y and z images
+// are the warp's, whole rows at a time; most rows have none.
 template <class S, bool CONTACT, int E>
 __device__ __forceinline__ void write_cells(const GridGeom &g, const Faces<typename Cell<S>::T> &fc, S *f,
                                             const Vec<S> &v, int i, int j, int k)

@@ -228,7 +228,7 @@ __device__ __forceinline__ bool in_band(float x)
 __device__ __forceinline__ bool in_band(double x) { return x > 1e-6 && x < 1.0 - 1e-6; }
 
 // the upper words of 1e-6 and 1 - 1e-6 bound those of the band's cells
-static_assert(0x3eb0c6f7u < 0x3feffffeu, "band limits");
+constexpr unsigned kBandLo = 0x3eb0c6f7u, kBandHi = 0x3feffffdu;
 // a double's bits as a signed integer of the same order (-0 below +0), and back
 __device__ __forceinline__ long long order_key(double x)
 {
@@ -548,7 +548,7 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
                             const long long k = order_key(x);
                             klo = k < klo ? k : klo;
                             khi = k > khi ? k : khi;
-                            if (h - 0x3eb0c6f7u <= 0x3feffffeu - 0x3eb0c6f7u) parts |= 1u << ((t * E + e) / 4);
+                            if (h - kBandLo <= kBandHi - kBandLo) parts |= 1u << ((t * E + e) / 4);
                         }
             }
             if constexpr (sizeof(R) == 4) {
@@ -662,7 +662,8 @@ __device__ __forceinline__ void stats_pass(const StatsArgs &a, const S *f, doubl
 }
 
 template <class S>
-__global__ void __launch_bounds__(256, sizeof(S) == 8 ? 2 : 3) stats_kernel(const StatsArgs a, const S *f, double *partials)
+__global__ void __launch_bounds__(256, sizeof(S) == 8 ? 2 : 3)
+    stats_kernel(const StatsArgs a, const S *f, double *partials)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     stats_pass<S>(a, f, partials + (long long)blockIdx.x * kNStat, blockIdx.x, gridDim.x);

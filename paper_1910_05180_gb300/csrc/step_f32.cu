@@ -9,7 +9,8 @@ cudaError_t launch_step_f32(const StepCoef<float> &c, const float *src, float *d
     if (cfg.mode & kImages) return launch_step_f32_img(c, src, dst, err, cfg, tma, which, st);
     if (cfg.rounding == SPFM_ROUND_STOCHASTIC) return launch_step_f32_sr(c, src, dst, err, cfg, tma, which, st);
     const CUtensorMap *map = f32_step_map(tma, which, c, cfg.scheme, src);
-    return launch_step_t<float, float, SPFM_F32_TX, SPFM_F32_TY, false, false, kSqTX, kSqTY>(c, src, dst, err, cfg, map, st);
+    return launch_step_t<float, float, SPFM_F32_TX, SPFM_F32_TY, false, false, kSqTX, kSqTY>(
+        c, src, dst, err, cfg, map, st);
 }
 
 size_t batch_grid_bytes_f32() { return sizeof(BatchGrid<float>); }

@@ -9,6 +9,7 @@ cudaError_t launch_step_f32_img(const StepCoef<float> &c, const float *src, floa
 {
     if (cfg.rounding == SPFM_ROUND_STOCHASTIC) return launch_step_f32_img_sr(c, src, dst, err, cfg, tma, which, st);
     const CUtensorMap *map = f32_step_map(tma, which, c, cfg.scheme, src);
-    return launch_step_t<float, float, SPFM_F32_TX, SPFM_F32_TY, true, false, kSqTX, kSqTY>(c, src, dst, err, cfg, map, st);
+    return launch_step_t<float, float, SPFM_F32_TX, SPFM_F32_TY, true, false, kSqTX, kSqTY>(
+        c, src, dst, err, cfg, map, st);
 }
 }  // namespace spfm

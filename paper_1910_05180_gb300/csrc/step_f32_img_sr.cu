@@ -9,6 +9,7 @@ cudaError_t launch_step_f32_img_sr(const StepCoef<float> &c, const float *src, f
                                    LaunchCfg cfg, TmaCache *tma, int which, cudaStream_t st)
 {
     const CUtensorMap *map = f32_step_map(tma, which, c, cfg.scheme, src);
-    return launch_step_t<float, float, SPFM_F32_TX, SPFM_F32_TY, true, true, kSqTX, kSqTY>(c, src, dst, err, cfg, map, st);
+    return launch_step_t<float, float, SPFM_F32_TX, SPFM_F32_TY, true, true, kSqTX, kSqTY>(
+        c, src, dst, err, cfg, map, st);
 }
 }  // namespace spfm

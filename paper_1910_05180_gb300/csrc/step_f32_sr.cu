@@ -9,7 +9,8 @@ cudaError_t launch_step_f32_sr(const StepCoef<float> &c, const float *src, float
                                TmaCache *tma, int which, cudaStream_t st)
 {
     const CUtensorMap *map = f32_step_map(tma, which, c, cfg.scheme, src);
-    return launch_step_t<float, float, SPFM_F32_TX, SPFM_F32_TY, false, true, kSqTX, kSqTY>(c, src, dst, err, cfg, map, st);
+    return launch_step_t<float, float, SPFM_F32_TX, SPFM_F32_TY, false, true, kSqTX, kSqTY>(
+        c, src, dst, err, cfg, map, st);
 }
 
 cudaError_t launch_batch_f32_sr(const void *grids, BatchList list, int parity, int *err,

@@ -16,12 +16,12 @@
 // Boundary conditions.  The kernel reads the ghost layer.  In general it
 // writes interior cells only and a face kernel (boundary.cu) refreshes the
 // ghosts of the new field after each step.  When every face is periodic and a
-// row is a whole number of 32-byte sectors, the ghosts are plain periodic images: the thread that writes a cell next to a face also
-// writes its image(s) on the far side (x images as whole 32-byte sectors of
-// the row pads, two threads a sector), so no face kernel runs; where no face is
-// periodic the producer warp builds the ghosts of the planes it stages.  The
-// kernels of a call chain by programmatic dependent launch, each waiting for
-// the one before in every tile.
+// row is a whole number of 32-byte sectors, the ghosts are plain periodic images:
+// the thread that writes a cell next to a face also writes its image(s) on the
+// far side (x images as whole 32-byte sectors of the row pads, two threads a
+// sector), so no face kernel runs; where no face is periodic the producer warp
+// builds the ghosts of the planes it stages.  The kernels of a call chain by
+// programmatic dependent launch, each waiting for the one before in every tile.
 //
 // Arithmetic.  From each plane every thread forms, for its cells,
 //   C  = phi at the cell,
@@ -149,7 +149,7 @@ struct PackCoef {
     using P = typename PackT<T>::P;
     P one, m2, m4, c1, c2, c3, ct, nkmu, nkap;
     // coefficients of q^i in -dt N and in D, side by side (one 16- or 32-byte
-    // load: a batch reads them from its grid records in global memory)
+    // load: a batch reads them from its warps' copies in shared memory)
     struct __align__(2 * sizeof(P)) Ratio {
         P num, den;
     };
@@ -1266,8 +1266,8 @@ struct BatchGrid {
 // producer warp stages the ghosts of the faces; no ghost kernel runs).
 template <class S, class T, int STENCIL, int KIND, int TX, int TY, bool SQ, bool SR = false>
 __global__ void __launch_bounds__(TileShape<S, T, TX, TY>::NTHREADS, kBatchCtasPerSm)
-    spfm_batch_kernel(const BatchGrid<T> *__restrict__ grids, const BatchList list, int parity, int *__restrict__ err, const long long *__restrict__ steps,
-                      int sub, int fwd)
+    spfm_batch_kernel(const BatchGrid<T> *__restrict__ grids, const BatchList list, int parity,
+                      int *__restrict__ err, const long long *__restrict__ steps, int sub, int fwd)
 {
     using Sh = TileShape<S, T, TX, TY>;
     __shared__ __align__(128) S stages[Sh::NS * Sh::STAGE];
@@ -1291,7 +1291,8 @@ __global__ void __launch_bounds__(TileShape<S, T, TX, TY>::NTHREADS, kBatchCtasP
         const BatchItem it = list.work[w];
         const BatchGrid<T> &bg = grids[it.grid];
         const int cur = bg.cur ^ parity;
-        const CUtensorMap *map = SQ ? (bg.has_map_sq ? &bg.map_sq[cur] : nullptr) : (bg.has_map ? &bg.map[cur] : nullptr);
+        const CUtensorMap *map =
+            SQ ? (bg.has_map_sq ? &bg.map_sq[cur] : nullptr) : (bg.has_map ? &bg.map[cur] : nullptr);
         if (map && threadIdx.x == Sh::NCONS)
             asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(map) : "memory");
         const bool last = w + 1 == end;
@@ -1437,7 +1438,8 @@ cudaError_t launch_step_t(const StepCoef<T> &c, const S *src, S *dst, int *err, 
         return cudaLaunchKernelEx(&lc, kern, c, pc, src, dst, err, zchunk, map, use, mode);
     };
     cudaError_t le = cudaSuccess;
-#define SPFM_LAUNCH(ST, KD) le = go(spfm_step_kernel<S, T, ST, KD, TX, TY, R, IMG, SR>, TileShape<S, T, TX, TY, R>::NTHREADS)
+#define SPFM_LAUNCH(ST, KD) \
+    le = go(spfm_step_kernel<S, T, ST, KD, TX, TY, R, IMG, SR>, TileShape<S, T, TX, TY, R>::NTHREADS)
 #define SPFM_BY_KIND(ST)                        \
     do {                                        \
         if (kind == 0) SPFM_LAUNCH(ST, 0);      \
