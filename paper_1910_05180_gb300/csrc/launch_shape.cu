@@ -14,31 +14,33 @@
 // - Few rounds: every chunk length from 4 to 64 planes is scored by the
 //   makespan of a greedy dispatch of the CTAs, in launch order, to the slots:
 //   a CTA takes (its planes + 1) units, and one that has to wait for a slot
-//   2 units more (the next step's CTAs, launched early, compete for the slots
-//   that free up).  The shortest makespan wins, ties to the longer chunk.
-//   The launch order puts the short last chunk of each column last.  Fitted
-//   to sweeps of 4 ... 48 planes (FP32, 96^3 ... 384^3, contact and periodic
-//   faces, CF / TI / TI_n / stochastic rounding, 19 configurations): the
-//   choice ran 1.5 % above the best measured one on average, 10 % at worst,
-//   where chunks of 16 planes or more lost up to 2x on grids of 96^3 ... 192^3.
-//   The model takes a CTA's speed as independent of the CTAs beside it on its
-//   SM, which holds for the streaming kernels at three or four CTAs per SM;
-//   kernels with fewer keep the rule of many rounds.
-//
+//   2 units more (its start and the fill of its ring, which a CTA of the first
+//   round overlaps with the launch before; both constants are a fit).  The
+//   shortest makespan wins, ties to the longer chunk.  The launch order puts the
+//   short last chunk of each column last.  The model takes a CTA's speed as
+//   independent of the CTAs beside it on its SM, which holds for the streaming
+//   kernels at three or four CTAs per SM; a kernel with fewer (none of this
+//   family) would keep the rule of many rounds.
 // - Less than a round at 4 planes: the shortest chunks that still fit one round,
 //   since such a launch lasts as long as one CTA's march (FP32, contact faces, 13
-//   groups, us a step: 32^3 4 planes 7.6, 1 (chosen) 5.2; 64^3 7.6 and 5.4; 96^3
-//   4 planes 8.0, 3 (chosen) 7.6, 2 (more than a round) 9.9).
+//   groups, us a step: 32^3 4 planes 7.1, 1 (chosen) 4.9; 64^3 7.0 and 4.8; 96^3
+//   4 planes 7.5, 3 (chosen) 7.1, 2 (more than a round) 9.7).
+//
+// Sweeps of 1 to 64 planes over 40 streaming launches (FP32 32^3 to 384^3, periodic,
+// contact and mixed faces, TI, CF and stochastic rounding, 150 x 133 x 117; BF16
+// 128^3 and 256^3): the choice ran 1.0 % above the best measured one on average
+// and 10 % at worst (320^3 channel: 54 planes 59.6 us, 18 planes 54.1); at 320^3
+// and 384^3 otherwise 3 to 5 %.
 //
 // TI_n has a rule of its own: its CTAs differ in work (those in the interface
 // band compute the 13 couplings of each cell, a plane of them some 2 us; those
 // in the bulk do not), so it wants many small CTAs.  About six rounds of
 // the slots, chunks of 4 to 16 planes; where chunks of 4 leave slots empty, the
 // shortest chunks that still fit one round.  Measured at two CTAs per SM (us a
-// step, FP32 27-point, planes per CTA): 60^3 cube 20: 37.9, 4: 12.6, 1 (chosen):
-// 10.1; 64^3 plane all in the band 16: 40.0, 4: 13.8, 1 (chosen): 7.4; 96^3 16:
-// 46.2, 4 (chosen): 15.5, 2: 16.3; 192^3 16: 72, 4 (chosen): 60.5, 2: 69.8;
-// 256^3 16: 96.0, 8: 90.4 (9 chosen), 4: 94.2; 320^3 16 (chosen): 124.6, 8: 129.
+// step, FP32 27-point, tilted plane, planes per CTA): 60^3 20: 34.3, 4: 10.1, 1
+// (chosen): 7.0; 64^3 16: 28.9, 4: 8.9, 1 (chosen): 5.2; 96^3 16: 29.1, 4 (chosen):
+// 12.7, 2: 14.0; 192^3 16: 65.9, 4 (chosen): 54.1, 2: 57.1; 256^3 16: 113.6, 9
+// (chosen): 106.1, 6: 104.6; 320^3 16 (chosen): 178.2, 12: 171.7, 4: 183.0.
 //
 // The FP64 kernels (CF and TI global) are bound by the FP64 pipe, which the CTAs
 // of an SM share: what counts is the work of the fullest SM, ceil(CTAs / SMs)
@@ -46,9 +48,10 @@
 // and 21 more as it is written (the halo planes are only read).  A CTA alone on
 // its SM leaves the pipe idle a fifth of the time, two leave it 2 %.  Chunks of
 // 1 to 64 planes, the least work, ties to the longer chunk.  Measured, us a step
-// (planes per CTA): 128 x 32 x 32 7-point 2 (chosen) 10.6, 1: 15.0, 4 (the
-// streaming rule) 15.8; 72^3 4 (chosen) 81, 2: 100; 96^3 6 (chosen) 107, 12: 126,
-// 2: 125; 100^3 10 (chosen) 167, 5: 225; 256^3 37 (chosen) 1047, 16: 1066.
+// (planes per CTA; 13 groups but for the first): 128 x 32 x 32 7-point 2 (chosen)
+// 10.9, 1: 11.7, 4 (the streaming rule) 17.4; 72^3 4 (chosen) 66, 2: 97; 96^3 6
+// (chosen) 95, 12: 109, 2: 109; 100^3 10 (chosen) 153, 5: 219; 256^3 37 (chosen)
+// 1632, 16: 1669.
 #include <map>
 #include <mutex>
 #include <queue>
