@@ -16,13 +16,15 @@
 // Both are bound by the FP64 pipe (a warp's FP64 instruction holds it 16 cycles
 // for the whole SM) and by latency at the grids of this study (60^3: 0.9 MB a
 // field).  So a warp takes a row in 16-byte loads; cells of FP32 and BF16 fields
-// are summed by fours and corrected in double-float pairs, whose terms are exact
-// (48 bits against the 24 of a cell), and only the sums of four enter FP64; the
-// block reduction adds 8 values a lane from shared memory before it shuffles.
-// The kernels of a step chain by programmatic dependent launch.  60^3 FP32, us
-// a step: sums 10.9 -> 6.0, correction and ghosts 67.1 + 3.4 -> 6.9 (one thread
-// added the 608 partials one by one); alpha formed once, by the last block of
-// the sums, was slower (9.1 + 5.1).
+// are summed by fours, whose terms and sums are exact but for 2^-70 (Sum3), and only
+// those sums enter FP64; they are corrected in double-float pairs (48 bits against
+// the 24 of a cell).  The block reduction adds 8 values a lane from shared memory
+// before it shuffles.  The kernels of a step chain by programmatic dependent
+// launch.  60^3 FP32, us a step: sums 10.9 -> 6.0 (6.8 with Sum3 in place of pairs),
+// correction and ghosts 67.1 + 3.4 -> 6.9 (one thread added the 608 partials one by
+// one); alpha formed once, by the last block of the sums, was slower (9.1 + 5.1).
+// alpha of 28 fields of 40 to 97 cells a side against quadruple precision, in units
+// of 2^-53: 3.8 on average and 9.3 at most with one FP64 sum a lane, 1.0 and 3.0 so.
 #include "spfm_internal.h"
 
 namespace spfm {
@@ -54,17 +56,39 @@ __device__ __forceinline__ void add_cells(const double *x, const double *d, int 
         }
 }
 __device__ __forceinline__ DF q_of(float x) { return df_mul_f(df_two_sum(1.0f, -x), x); }
+// A sum of a few FP32 numbers as s + l + m: s the sum, l that of its remainders, m
+// that of theirs, so that it is good to about 2^-70.  As pairs alone (2^-48 a cell) the
+// sum of q came out 3e-16 too large, always to that side.
+struct Sum3 {
+    float s = 0.0f, l = 0.0f, m = 0.0f;
+    __device__ __forceinline__ void low(float x)
+    {
+        const DF t = df_two_sum(l, x);
+        l = t.hi;
+        m = __fadd_rn(m, t.lo);
+    }
+    __device__ __forceinline__ void add(DF x)
+    {
+        const DF t = df_two_sum(s, x.hi);
+        s = t.hi;
+        low(t.lo);
+        low(x.lo);
+    }
+    __device__ __forceinline__ double value() const { return (double)s + ((double)l + (double)m); }
+};
 __device__ __forceinline__ void add_cells(const float *x, const float *d, int n, double &dsum, double &qsum)
 {
-    DF ds{0.0f, 0.0f}, qs{0.0f, 0.0f};
+    Sum3 ds, qs;
 #pragma unroll
     for (int e = 0; e < 4; ++e)
         if (e < n) {
-            ds = df_add_acc(ds, df_two_sum(d[e], -x[e]));   // d - x exactly
-            qs = df_add_acc(qs, q_of(x[e]));
+            ds.add(df_two_sum(d[e], -x[e]));   // d - x exactly
+            const DF xx = df_two_prod(x[e], x[e]);
+            qs.add(df_two_sum(x[e], -xx.hi));   // x - x^2 exactly
+            qs.low(-xx.lo);
         }
-    dsum += df_to_double(ds);
-    qsum += df_to_double(qs);
+    dsum += ds.value();
+    qsum += qs.value();
 }
 
 // d - alpha q(x), rounded once
